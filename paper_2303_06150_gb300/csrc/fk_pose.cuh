@@ -17,8 +17,8 @@
 // each atom's owner; each bond's parent (the owner of its moving endpoint v,
 // which no other bond's list holds); the bonds in decreasing moving-side
 // size (a parent before its children) and grouped by depth in the bond
-// tree; the bond axes. fk_table_kernel runs it once per ligand and writes
-// the result out, with the atoms listed by owner; the scoring and gradient
+// tree; the bond axes. The packer writes the same values out once per ligand
+// (the table, with the atoms listed by owner); the scoring and gradient
 // kernels stage it with fk_load (vector copies). Transforms are 12 floats:
 // three rows (m0 m1 m2 | o).
 #pragma once
@@ -155,12 +155,11 @@ __device__ inline bool fk_stage(const Packed& pk, int a0, int N, int r0, int n, 
 }
 
 // Stage ligand l = (a0, N, r0, n) for the warp (all 32 lanes call it) from
-// the forward-kinematics table (pk.fk_*, written by fk_table_kernel with
-// fk_stage<true>): the contents fk_stage<true> builds, but for the
-// moving-atom lists (nothing reads them after staging), with the atoms
-// listed by owner (S.sx, S.own in the table's order) and S.sb[b].y the list
-// position of bond b's v (S.sb[b].x unused). Vector copies, no per-bond
-// passes. Returns false, on every lane, when the table marks the ligand's
+// the forward-kinematics table (pk.fk_*, written by the packer): the
+// contents fk_stage<true> builds, but for the moving-atom lists (nothing
+// reads them after staging), with the atoms listed by owner (S.sx, S.own in
+// the table's order) and S.sb[b].y the list position of bond b's v (S.sb[b].x
+// unused). Vector copies, no per-bond passes. Returns false, on every lane, when the table marks the ligand's
 // lists as malformed.
 __device__ inline bool fk_load(const Packed& pk, int l, int a0, int N, int r0, int n, const FkLigand& S, int lane) {
   static_assert(kFkLoffBytes == 48 && kFkBad > LIGEN_MAX_ROT, "depth row of the table = the staged row");

@@ -21,7 +21,7 @@ struct LigandsDev {
   const int32_t* rot_edge;
 };
 
-// Packer outputs.
+// Packer outputs; a NULL one is not written.
 struct Packed {
   float4* xc;        // [sum N] centred input coordinates; w = atom type (int bits)
   uchar4* binfo;     // [sum n] (fixed u, moving v, moving atoms excluding v, 0)
@@ -32,8 +32,8 @@ struct Packed {
   int32_t* axis;     // [sum n][2] optional: (u, v)
   uint32_t* touch;   // [sum n] optional: bit b of touch[b'] set when turning bond b'
                      // moves an atom bond b's sweep reads (bit b' always set)
-  // Forward-kinematics table (fk_table_kernel; read by the pose-per-lane
-  // scoring and pose-group gradient kernels), optional. A ligand's atoms
+  // Forward-kinematics table (all NULL or none; read by the pose-per-lane
+  // scoring and pose-group gradient kernels). A ligand's atoms
   // are listed by owner (bond 0's, bond 1's, ..., then the root frame's;
   // input order within an owner):
   float4* fk_xs;     // [sum N] centred input coordinates (w = type) in that order
@@ -163,10 +163,9 @@ cudaError_t launch_grid_prep(const float* values, int nx, int ny, int nz, int nc
 // Records in format `fmt` (RecFormat) for the docking kernel.
 cudaError_t launch_grid_prep_fmt(const float* values, int nx, int ny, int nz, int nc, int fmt, void* rec,
                                  cudaStream_t s);
-cudaError_t launch_pack(const LigandsDev& lig, int nc, const Packed& out, cudaStream_t s);
-// The forward-kinematics table of every ligand (pk.fk_*), after launch_pack;
-// max_atoms / max_rot: the library's largest ligand.
-cudaError_t launch_fk_table(const LigandsDev& lig, const Packed& pk, int max_atoms, int max_rot, cudaStream_t s);
+// max_atoms: the library's largest ligand. With out.fk_xs set, the
+// forward-kinematics table (out.fk_*) too.
+cudaError_t launch_pack(const LigandsDev& lig, int nc, const Packed& out, int max_atoms, cudaStream_t s);
 size_t dock_smem_bytes(int max_atoms, int max_rot, int max_frag, int rpc);
 bool dock_lanes_supported(int lanes);
 bool dock_shape_supported(int lanes, int fmt);

@@ -1,7 +1,7 @@
 // Pose gradients and gradient refinement. Two kernels: grad_lane_kernel
 // (4 or more poses per ligand; the main path) puts a group of G = 1, 2 or 4
 // lanes on each pose and builds the torsions as forward kinematics
-// (fk_pose.cuh, the table of fk_table_kernel), the torsion gradients from
+// (fk_pose.cuh, the packer's table), the torsion gradients from
 // subtree sums, launched by rotatable-bond class; grad_kernel / refine_kernel
 // (fewer poses) put a group of kGradLanes lanes on each pose, 32 / kGradLanes
 // poses (of one ligand) per warp, and apply the torsions atom by atom. What

@@ -2,13 +2,11 @@
 // positions as the docking output defines them (torsions bond by bond in
 // index order on the centred input coordinates, each about the current axis
 // from its fixed endpoint to its moving endpoint; then R(q / |q|) and t).
-// Three kernels:
+// Two kernels:
 //   score_lane_kernel  16 or more poses per ligand: one pose per lane, the
-//                      torsions as forward kinematics (fk_pose.cuh), launched
-//                      by rotatable-bond class (see its comment);
-//   fk_table_kernel    the ligand-only part of the forward kinematics, once
-//                      per library or call (owners, parents, orders, axes,
-//                      the atoms listed by owner);
+//                      torsions as forward kinematics (fk_pose.cuh, the
+//                      packer's table), launched by rotatable-bond class
+//                      (see its comment);
 //   score_kernel       fewer poses: a group of kScoreLanes lanes per pose,
 //                      two poses of one ligand per warp, the torsions
 //                      applied atom by atom (pose_build.cuh). Measured on
@@ -264,69 +262,7 @@ cudaError_t config_sl(const ScoreArgs& a, LaunchCfg* c) {
   return cudaSuccess;
 }
 
-// One warp per ligand: the ligand staged as fk_stage<true> stages it, then
-// the parts the scoring and gradient kernels read (owners, parents, orders,
-// depth offsets, axes) written to the table, with the malformed flag.
-constexpr int kTabWarps = 4;
-
-__global__ void __launch_bounds__(32 * kTabWarps) fk_table_kernel(const LigandsDev lig, const Packed pk, int acap,
-                                                                  int ncap) {
-  extern __shared__ __align__(16) unsigned char tab_smem[];
-  const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int l = blockIdx.x * kTabWarps + w;
-  if (l >= lig.L) return;   // uniform over the warp
-  const size_t lig_bytes = fk_ligand_carve(acap, ncap, nullptr, nullptr);
-  const size_t per = lig_bytes + LIGEN_MAX_ATOMS;   // + each atom's position in the owner-ordered list
-  FkLigand S;
-  fk_ligand_carve(acap, ncap, tab_smem + (size_t)w * per, &S);
-  uint8_t* pos = tab_smem + (size_t)w * per + lig_bytes;
-  uint8_t* row = pk.fk_loff + (size_t)l * kFkLoffBytes;
-  const int a0 = lig.atom_off[l], N = lig.atom_off[l + 1] - a0;
-  const int r0 = lig.rot_off[l], n = lig.rot_off[l + 1] - r0;
-  bool ok = pk.status[l] == 0 && N >= 1 && N <= acap && n >= 0 && n <= ncap;
-  if (ok) ok = fk_stage<true>(pk, a0, N, r0, n, S, lane);
-  if (!ok) {   // nothing of the ligand is read: only the flag
-    if (lane < kFkLoffBytes) row[lane] = lane == kFkBad ? 1 : 0;
-    if (lane + 32 < kFkLoffBytes) row[lane + 32] = lane + 32 == kFkBad ? 1 : 0;
-    return;
-  }
-  // the atoms listed by owner (bond 0's, ..., bond n-1's, the root's; a
-  // stable counting sort), so that a pose's consecutive atoms mostly share
-  // one transform
-  if (lane == 0) {
-    int start[LIGEN_MAX_ROT + 2];
-    for (int o = 0; o <= n + 1; ++o) start[o] = 0;
-    for (int i = 0; i < N; ++i) ++start[S.own[i] + 1];
-    for (int o = 0; o < n + 1; ++o) start[o + 1] += start[o];
-    for (int i = 0; i < N; ++i) pos[i] = (uint8_t)start[S.own[i]]++;
-  }
-  __syncwarp();
-  for (int i = lane; i < N; i += 32) {
-    pk.fk_xs[a0 + pos[i]] = S.sx[i];
-    pk.fk_own[a0 + pos[i]] = S.own[i];
-  }
-  for (int b = lane; b < n; b += 32) {
-    pk.fk_ax[r0 + b] = S.ax[b];
-    pk.fk_bond[r0 + b] = make_uchar4(S.par[b], S.ord[b], S.lord[b], pos[S.sb[b].y]);
-  }
-  const int depths = S.loff[LIGEN_MAX_ROT];
-  for (int k = lane; k < kFkLoffBytes; k += 32)
-    row[k] = k <= depths || k == LIGEN_MAX_ROT ? S.loff[k] : 0;   // k == kFkBad: 0
-}
-
 }  // namespace
-
-cudaError_t launch_fk_table(const LigandsDev& lig, const Packed& pk, int max_atoms, int max_rot, cudaStream_t s) {
-  if (lig.L == 0) return cudaSuccess;
-  const size_t smem = (size_t)kTabWarps * (fk_ligand_carve(max_atoms, max_rot, nullptr, nullptr) + LIGEN_MAX_ATOMS);
-  if (smem > 48 * 1024) {
-    cudaError_t e = cudaFuncSetAttribute(fk_table_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-  }
-  const unsigned blocks = (unsigned)((lig.L + kTabWarps - 1) / kTabWarps);
-  fk_table_kernel<<<blocks, 32 * kTabWarps, smem, s>>>(lig, pk, max_atoms, max_rot);
-  return cudaGetLastError();
-}
 
 // One lane per pose. Measured on GB300, scoring the 600,000 kept screening
 // poses: 0.255 ms with 1 lane per pose, 0.275 ms with 2 (one transform set

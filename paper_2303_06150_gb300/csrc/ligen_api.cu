@@ -1001,7 +1001,7 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     float* coef = ar.at<float>(o_coef);
     LG_CUDA(launch_grid_prep_fmt(gvals, grid->nx, grid->ny, grid->nz, grid->nc, fmt, coef, s));
     tm.mark();
-    if (site == 0) LG_CUDA(launch_pack(lig, grid->nc, pk, s));
+    if (site == 0) LG_CUDA(launch_pack(lig, grid->nc, pk, sh.max_atoms, s));
     tm.mark();
 
     float* d_poses = ohost ? ar.at<float>(o_poses) : site_poses;
@@ -1178,10 +1178,10 @@ int ligen_score_poses(const ligen_ligands_t* ligands, const ligen_grid_t* grid, 
   const size_t o_coef = ar.take(grid_coef_bytes(grid));
   const size_t o_xc = ar.take(16 * (size_t)sh.atoms);
   const size_t o_binfo = ar.take(4 * (size_t)sh.rot);
-  const size_t o_frag = ar.take((size_t)kFragStride * sh.rot);
+  const bool lanes = poses_per_ligand >= kLanePosesMin;
+  const size_t o_frag = lanes ? 0 : ar.take((size_t)kFragStride * sh.rot);   // the table replaces the lists
   const size_t o_status = ar.take(4 * (size_t)L);
   const size_t o_list = ar.take(4 * plan.list.size());
-  const bool lanes = poses_per_ligand >= kLanePosesMin;
   const FkRegions o_fk = lanes ? take_fk(ar, sh, L) : FkRegions{};
   size_t o_poses = 0, o_scores = 0;
   if (ohost) {
@@ -1211,13 +1211,10 @@ int ligen_score_poses(const ligen_ligands_t* ligands, const ligen_grid_t* grid, 
   Packed pk{};
   pk.xc = ar.at<float4>(o_xc);
   pk.binfo = ar.at<uchar4>(o_binfo);
-  pk.frag = ar.at<uint8_t>(o_frag);
+  pk.frag = lanes ? nullptr : ar.at<uint8_t>(o_frag);
   pk.status = ar.at<int32_t>(o_status);
-  LG_CUDA(launch_pack(lig, grid->nc, pk, s));
-  if (lanes) {
-    set_fk(ar, o_fk, &pk);
-    LG_CUDA(launch_fk_table(lig, pk, sh.max_atoms, sh.max_rot, s));
-  }
+  if (lanes) set_fk(ar, o_fk, &pk);
+  LG_CUDA(launch_pack(lig, grid->nc, pk, sh.max_atoms, s));
   ScoreArgs sa{};
   sa.lig = lig;
   sa.pk = pk;
@@ -1323,8 +1320,7 @@ int ligen_prepare_scoring(const ligen_ligands_t* ligands, const ligen_grid_t* gr
       ce = cudaMemcpyAsync(h->d_list, h->plan.list.data(), 4 * (size_t)L, cudaMemcpyHostToDevice, s);
   }
   if (ce == cudaSuccess) ce = launch_grid_prep(gvals, grid->nx, grid->ny, grid->nz, grid->nc, h->coef, s);
-  if (ce == cudaSuccess && L) ce = launch_pack(lig, grid->nc, h->pk, s);
-  if (ce == cudaSuccess && L) ce = launch_fk_table(lig, h->pk, sh.max_atoms, sh.max_rot, s);
+  if (ce == cudaSuccess && L) ce = launch_pack(lig, grid->nc, h->pk, sh.max_atoms, s);
   if (ce != cudaSuccess) return bail(cuda_fail(ce, "preparing the scoring inputs"));
   // Host inputs are copied through the workspace asynchronously: wait for
   // the copies, so the caller may reuse its host buffers on return.
@@ -1441,10 +1437,10 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
   const size_t o_coef = ar.take(grid_coef_bytes(grid));
   const size_t o_xc = ar.take(16 * (size_t)sh.atoms);
   const size_t o_binfo = ar.take(4 * (size_t)sh.rot);
-  const size_t o_frag = ar.take((size_t)kFragStride * sh.rot);
+  const bool lanes = poses_per_ligand >= kGradLanePosesMin;
+  const size_t o_frag = lanes ? 0 : ar.take((size_t)kFragStride * sh.rot);   // the table replaces the lists
   const size_t o_status = ar.take(4 * (size_t)L);
   ScorePlan plan;   // ligands by rotatable-bond class for the pose-group kernel
-  const bool lanes = poses_per_ligand >= kGradLanePosesMin;
   if (lanes) plan_score(ligands->h_rot_off, L, &plan);
   const size_t o_list = ar.take(4 * plan.list.size());
   const FkRegions o_fk = lanes ? take_fk(ar, sh, L) : FkRegions{};
@@ -1476,13 +1472,10 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
   Packed pk{};
   pk.xc = ar.at<float4>(o_xc);
   pk.binfo = ar.at<uchar4>(o_binfo);
-  pk.frag = ar.at<uint8_t>(o_frag);
+  pk.frag = lanes ? nullptr : ar.at<uint8_t>(o_frag);
   pk.status = ar.at<int32_t>(o_status);
-  LG_CUDA(launch_pack(lig, grid->nc, pk, s));
-  if (lanes) {
-    set_fk(ar, o_fk, &pk);
-    LG_CUDA(launch_fk_table(lig, pk, sh.max_atoms, sh.max_rot, s));
-  }
+  if (lanes) set_fk(ar, o_fk, &pk);
+  LG_CUDA(launch_pack(lig, grid->nc, pk, sh.max_atoms, s));
   GradArgs ga{};
   ga.lig = lig;
   ga.pk = pk;
@@ -1567,31 +1560,27 @@ int ligen_pack_ligands(const ligen_ligands_t* ligands, int32_t n_channels, uint3
   Arena ar;
   LigandPlan lp;
   plan_ligands(ar, ligands, sh, lhost == 1, &lp);
-  const size_t o_xc = ar.take(16 * (size_t)sh.atoms);
-  const size_t o_binfo = ar.take(4 * (size_t)sh.rot);
-  const size_t o_frag = ar.take((size_t)kFragStride * sh.rot);
-  const size_t o_status = ar.take(4 * (size_t)L);
-  const size_t o_bucket = ar.take(4 * (size_t)L);
-  const size_t o_bits = ar.take(32 * (size_t)sh.rot);
-  const size_t o_axis = ar.take(8 * (size_t)sh.rot);
-  if ((rc = get_workspace(s, ar.used, &ar.base)) != LIGEN_OK) return rc;
+  // device outputs are written in place, host outputs through the workspace
+  const size_t o_status = ohost && status ? ar.take(4 * (size_t)L) : 0;
+  const size_t o_bucket = ohost && bucket ? ar.take(4 * (size_t)L) : 0;
+  const size_t o_bits = ohost && frag_bits ? ar.take(32 * (size_t)sh.rot) : 0;
+  const size_t o_axis = ohost && axis ? ar.take(8 * (size_t)sh.rot) : 0;
+  if (ar.used && (rc = get_workspace(s, ar.used, &ar.base)) != LIGEN_OK) return rc;
   LigandsDev lig;
   if ((rc = stage_ligands(ar, ligands, sh, lp, s, &lig)) != LIGEN_OK) return rc;
   Packed pk{};
-  pk.xc = ar.at<float4>(o_xc);
-  pk.binfo = ar.at<uchar4>(o_binfo);
-  pk.frag = ar.at<uint8_t>(o_frag);
-  pk.status = ar.at<int32_t>(o_status);
-  pk.bucket = ar.at<int32_t>(o_bucket);
-  pk.fbits = ar.at<uint32_t>(o_bits);
-  pk.axis = ar.at<int32_t>(o_axis);
-  LG_CUDA(launch_pack(lig, n_channels, pk, s));
-  const cudaMemcpyKind k = ohost ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
+  pk.status = ohost && status ? ar.at<int32_t>(o_status) : status;
+  pk.bucket = ohost && bucket ? ar.at<int32_t>(o_bucket) : bucket;
+  pk.fbits = ohost && frag_bits ? ar.at<uint32_t>(o_bits) : frag_bits;
+  pk.axis = ohost && axis ? ar.at<int32_t>(o_axis) : axis;
+  LG_CUDA(launch_pack(lig, n_channels, pk, sh.max_atoms, s));
+  if (!ohost) return LIGEN_OK;
+  const cudaMemcpyKind k = cudaMemcpyDeviceToHost;
   if (frag_bits && sh.rot) LG_CUDA(cudaMemcpyAsync(frag_bits, pk.fbits, 32 * (size_t)sh.rot, k, s));
   if (axis && sh.rot) LG_CUDA(cudaMemcpyAsync(axis, pk.axis, 8 * (size_t)sh.rot, k, s));
   if (bucket) LG_CUDA(cudaMemcpyAsync(bucket, pk.bucket, 4 * (size_t)L, k, s));
   if (status) LG_CUDA(cudaMemcpyAsync(status, pk.status, 4 * (size_t)L, k, s));
-  if (ohost) LG_CUDA(cudaStreamSynchronize(s));
+  LG_CUDA(cudaStreamSynchronize(s));
   return LIGEN_OK;
 }
 
@@ -1613,24 +1602,16 @@ int ligen_pack_touch(const ligen_ligands_t* ligands, int32_t n_channels, uint32_
   Arena ar;
   LigandPlan lp;
   plan_ligands(ar, ligands, sh, lhost == 1, &lp);
-  const size_t o_xc = ar.take(16 * (size_t)sh.atoms);
-  const size_t o_binfo = ar.take(4 * (size_t)sh.rot);
-  const size_t o_frag = ar.take((size_t)kFragStride * sh.rot);
-  const size_t o_status = ar.take(4 * (size_t)L);
-  const size_t o_touch = ar.take(4 * (size_t)sh.rot);
-  if ((rc = get_workspace(s, ar.used, &ar.base)) != LIGEN_OK) return rc;
+  const size_t o_touch = ohost ? ar.take(4 * (size_t)sh.rot) : 0;
+  if (ar.used && (rc = get_workspace(s, ar.used, &ar.base)) != LIGEN_OK) return rc;
   LigandsDev lig;
   if ((rc = stage_ligands(ar, ligands, sh, lp, s, &lig)) != LIGEN_OK) return rc;
   Packed pk{};
-  pk.xc = ar.at<float4>(o_xc);
-  pk.binfo = ar.at<uchar4>(o_binfo);
-  pk.frag = ar.at<uint8_t>(o_frag);
-  pk.status = ar.at<int32_t>(o_status);
-  pk.touch = ar.at<uint32_t>(o_touch);
-  LG_CUDA(launch_pack(lig, n_channels, pk, s));
-  LG_CUDA(cudaMemcpyAsync(touch, pk.touch, 4 * (size_t)sh.rot, ohost ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
-                          s));
-  if (ohost) LG_CUDA(cudaStreamSynchronize(s));
+  pk.touch = ohost ? ar.at<uint32_t>(o_touch) : touch;
+  LG_CUDA(launch_pack(lig, n_channels, pk, sh.max_atoms, s));
+  if (!ohost) return LIGEN_OK;
+  LG_CUDA(cudaMemcpyAsync(touch, pk.touch, 4 * (size_t)sh.rot, cudaMemcpyDeviceToHost, s));
+  LG_CUDA(cudaStreamSynchronize(s));
   return LIGEN_OK;
 }
 
@@ -1760,7 +1741,7 @@ int ligen_autotune(const ligen_ligands_t* ligands, const ligen_grid_t* grid, con
   pk.frag = ar.at<uint8_t>(o_frag);
   pk.touch = ar.at<uint32_t>(o_touch);
   pk.status = ar.at<int32_t>(o_status);
-  LG_CUDA(launch_pack(lig, grid->nc, pk, s));
+  LG_CUDA(launch_pack(lig, grid->nc, pk, sh.max_atoms, s));
   int32_t* d_order = ar.at<int32_t>(o_order);
   LG_CUDA(cudaMemcpyAsync(d_order, order.data(), 4 * order.size(), cudaMemcpyHostToDevice, s));
 
@@ -2010,7 +1991,7 @@ extern "C" int ligen_dock_batch_static(const ligen_ligands_t* ligands, const lig
   pk.frag = ar.at<uint8_t>(o_frag);
   pk.touch = ar.at<uint32_t>(o_touch);
   pk.status = ar.at<int32_t>(o_status);
-  LG_CUDA(launch_pack(lig, grid->nc, pk, s));
+  LG_CUDA(launch_pack(lig, grid->nc, pk, sh.max_atoms, s));
 
   DockArgs da{};
   da.lig = lig;
