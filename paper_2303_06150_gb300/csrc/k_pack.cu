@@ -199,6 +199,7 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(const LigandsDev 
       const int i = 32 * w + lane;
       x[w] = y[w] = z[w] = 0.f;
       ty[w] = ea[w] = eb[w] = 0;
+      if (32 * w >= N) continue;   // uniform
       if (i < N) {
         x[w] = lig.xyz[3 * (a0 + i)];
         y[w] = lig.xyz[3 * (a0 + i) + 1];
@@ -365,10 +366,11 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(const LigandsDev 
     }
     // moving-atom lists, owners (the shortest list holding the atom, the
     // first of equal ones) and touch masks, bond by bond
+    const bool lists = out.frag || out.touch || table;   // masks and axes alone need none of this
     unsigned key[W], touch = 1u << lane;
 #pragma unroll
     for (int w = 0; w < W; ++w) key[w] = 0xffffffc0u | n;
-    for (int b = 0; b < n; ++b) {
+    for (int b = 0; lists && b < n; ++b) {
       const unsigned mb = __shfl_sync(kFull, cnt, b);
       uint8_t* list = out.frag ? out.frag + (size_t)(r0 + b) * kFragStride : nullptr;
       unsigned hit = 0u;
