@@ -7,12 +7,26 @@
 // format (score, k, increments), so top-K, pose compaction and the FP64
 // re-score follow unchanged.
 //
-// One CTA per (ligand, restart). Threads take combination indices
-// c = ((k * nt + j_0) * nt + j_1) * nt + ... in a strided loop. Each pose is
-// rebuilt from the input conformation: the torsions are applied bond by bond
-// in index order, each about its axis as moved by the earlier bonds (the
-// axis endpoints are rotated first, then every atom), then the cube rotation
-// and the restart's orientation and translation.
+// An atom's position in a combination depends on k and on the increments of
+// the bonds that move it, not on the others: a bond that moves another
+// bond's axis moves that bond's whole list. So an atom moved by m of the n
+// bonds has n_theta^m energies per rotation, not n_theta^n, and they are
+// sampled once into a table in shared memory; a combination then costs one
+// table read and one subtraction per atom, in atom order, which gives the
+// same bits as rebuilding and sampling every atom of every combination.
+// Atoms go into the table by ascending m while kExTable entries hold them;
+// the ones that do not fit (many increments, deeply nested bonds) are
+// rebuilt per combination.
+//
+// A cluster of kExCluster CTAs takes one (ligand, restart), the rotations
+// split over its CTAs, and joins its winners through distributed shared
+// memory: without the split a call of a few hundred restarts leaves the
+// chip to the few ligands with the most bonds.
+// Measured on GB300, 97 ligands of 8-20 atoms and 0-3 bonds, 8 restarts, 30
+// degree steps, whole call: 2,780 us with every combination rebuilt by one
+// CTA per (ligand, restart), 242 us this way.
+#include <cooperative_groups.h>
+
 #include "../../include/ligen.h"
 #include "internal.h"
 
@@ -20,17 +34,138 @@ namespace ligen {
 namespace {
 
 constexpr int kExThreads = 128;
+constexpr int kExCluster = 8;     // CTAs per (ligand, restart): the portable maximum
+constexpr int kExTable = 6144;    // table entries: 24 KB, seven CTAs per SM with the rest
+constexpr int kExVec = 4;         // combinations a thread sums side by side
+constexpr uint16_t kExDirect = 0xffffu;
+
+// q / d for q < 2^27 by multiplication: m = ceil(2^40 / d) is off by less
+// than d / 2^40 relative to 1 / d, q * d < 2^40, and the product fits 64 bits
+// because q < n_rigid * d^4 and q < 2^27.
+struct ExDiv {
+  unsigned d;
+  unsigned long long m;
+  __device__ explicit ExDiv(unsigned dd) : d(dd), m(((1ull << 40) + dd - 1) / dd) {}
+  __device__ unsigned operator()(unsigned q) const { return d == 1 ? q : (unsigned)((q * m) >> 40); }
+};
+
+struct ExLigand {
+  float4 sx[LIGEN_MAX_ATOMS];
+  uint2 stride[LIGEN_MAX_ATOMS];    // table strides of bonds 0..3, 16 bits each
+  uint16_t base[LIGEN_MAX_ATOMS];   // first table entry, or kExDirect
+  uint8_t mask[LIGEN_MAX_ATOMS];    // bonds that move the atom
+  uint8_t slot[LIGEN_MAX_ATOMS];    // tabled atoms by first entry
+  int axis[kExMaxRot][2];
+  int n_slots, entries;
+};
+
+// Bond b's axis after the earlier bonds of `use` with increments j: moving
+// end pv, unit direction kd, and the turn's cosine and sine.
+__device__ __forceinline__ void ex_axes(const ExLigand& S, unsigned use, int n, const int (&j)[kExMaxRot], int step_deg,
+                                        float (&pv)[kExMaxRot][3], float (&kd)[kExMaxRot][3], float (&cs)[kExMaxRot],
+                                        float (&sn)[kExMaxRot]) {
+#pragma unroll
+  for (int b = 0; b < kExMaxRot; ++b) {
+    if (b >= n) break;
+    if (!(use >> b & 1u)) continue;
+    const int iu = S.axis[b][0], iv = S.axis[b][1];
+    float pu[3] = {S.sx[iu].x, S.sx[iu].y, S.sx[iu].z};
+    float pw[3] = {S.sx[iv].x, S.sx[iv].y, S.sx[iv].z};
+#pragma unroll
+    for (int e = 0; e < kExMaxRot; ++e) {
+      if (e >= b) break;
+      if (!(use >> e & 1u)) continue;
+      if (S.mask[iu] >> e & 1u) rodrigues_apply(pu, pv[e], kd[e], cs[e], sn[e]);
+      if (S.mask[iv] >> e & 1u) rodrigues_apply(pw, pv[e], kd[e], cs[e], sn[e]);
+    }
+    const float d0 = pw[0] - pu[0], d1 = pw[1] - pu[1], d2 = pw[2] - pu[2];
+    const float inv = rsqrtf(d0 * d0 + d1 * d1 + d2 * d2);
+    kd[b][0] = d0 * inv; kd[b][1] = d1 * inv; kd[b][2] = d2 * inv;
+    pv[b][0] = pw[0]; pv[b][1] = pw[1]; pv[b][2] = pw[2];
+    torsion_cs(j[b], step_deg, &cs[b], &sn[b]);
+  }
+}
+
+// Energy of atom i, turned by the bonds of its mask, under the rotation and
+// scaling Mk and the offset o.
+template <int FMT>
+__device__ __forceinline__ float ex_energy(const DockArgs& a, const ExLigand& S, int i, int n, const float* Mk,
+                                           const float* o, const float (&pv)[kExMaxRot][3],
+                                           const float (&kd)[kExMaxRot][3], const float (&cs)[kExMaxRot],
+                                           const float (&sn)[kExMaxRot]) {
+  const float4 X = S.sx[i];
+  float y[3] = {X.x, X.y, X.z};
+#pragma unroll
+  for (int b = 0; b < kExMaxRot; ++b) {
+    if (b >= n) break;
+    if (S.mask[i] >> b & 1u) rodrigues_apply(y, pv[b], kd[b], cs[b], sn[b]);
+  }
+  const float ux = fmaf(Mk[0], y[0], fmaf(Mk[1], y[1], fmaf(Mk[2], y[2], o[0])));
+  const float uy = fmaf(Mk[3], y[0], fmaf(Mk[4], y[1], fmaf(Mk[5], y[2], o[1])));
+  const float uz = fmaf(Mk[6], y[0], fmaf(Mk[7], y[1], fmaf(Mk[8], y[2], o[2])));
+  return grid_sample_fmt<FMT>(a.grid, ux, uy, uz, __float_as_int(X.w));
+}
+
+// Best of `total` combinations that start at combination c0 of the search
+// (whole rotations; the table holds them), all atoms tabled. NB >= n.
+template <int NB>
+__device__ __forceinline__ void ex_sum(const ExLigand& S, const float* tab, int N, int n, const ExDiv& by_nt,
+                                       unsigned total, long long c0, float& best, long long& bestc) {
+  for (unsigned t = threadIdx.x; t < total; t += kExThreads * kExVec) {
+    unsigned off[kExVec];
+    unsigned j[kExVec][NB];
+    float acc[kExVec];
+#pragma unroll
+    for (int v = 0; v < kExVec; ++v) {
+      unsigned q = min(t + v * kExThreads, total - 1);
+#pragma unroll
+      for (int b = NB - 1; b >= 0; --b) {
+        j[v][b] = 0u;
+        if (b < n) {
+          const unsigned up = by_nt(q);
+          j[v][b] = q - up * by_nt.d;
+          q = up;
+        }
+      }
+      off[v] = q * S.entries;
+      acc[v] = 0.f;
+    }
+    for (int i = 0; i < N; ++i) {
+      const uint2 s = S.stride[i];
+      const unsigned base = S.base[i];
+#pragma unroll
+      for (int v = 0; v < kExVec; ++v) {
+        unsigned at = base + off[v] + j[v][0] * (s.x & 0xffffu);
+        if constexpr (NB > 1) at += j[v][1] * (s.x >> 16);
+        if constexpr (NB > 2) at += j[v][2] * (s.y & 0xffffu);
+        if constexpr (NB > 3) at += j[v][3] * (s.y >> 16);
+        acc[v] -= tab[at];
+      }
+    }
+#pragma unroll
+    for (int v = 0; v < kExVec; ++v)   // t ascends per thread: ties keep the first
+      if (t + v * kExThreads < total && acc[v] > best) {
+        best = acc[v];
+        bestc = c0 + t + v * kExThreads;
+      }
+  }
+}
 
 template <int FMT>
-__global__ void __launch_bounds__(kExThreads) exhaustive_kernel(const DockArgs a) {
-  __shared__ float4 sx[LIGEN_MAX_ATOMS];
-  __shared__ uint32_t member[kExMaxRot][LIGEN_MAX_ATOMS / 32];
-  __shared__ int saxis[kExMaxRot][2];
+__global__ void __cluster_dims__(kExCluster, 1, 1) __launch_bounds__(kExThreads)
+    exhaustive_kernel(const DockArgs a, long long first) {
+  namespace cg = cooperative_groups;
+  __shared__ ExLigand S;
+  __shared__ float tab[kExTable];
   __shared__ float red_s[kExThreads / 32];
   __shared__ long long red_c[kExThreads / 32];
+  __shared__ float cta_s;
+  __shared__ long long cta_c;
 
-  const int l = blockIdx.x / a.R, r = blockIdx.x % a.R;
-  if (a.pk.status[l] != 0) return;   // uniform over the CTA
+  const long long item = first + blockIdx.x / kExCluster;
+  const int rank = blockIdx.x % kExCluster;
+  const int l = (int)(item / a.R), r = (int)(item % a.R);
+  if (a.pk.status[l] != 0) return;   // uniform over the cluster
   const int tid = threadIdx.x;
   const int a0 = a.lig.atom_off[l];
   const int N = a.lig.atom_off[l + 1] - a0;
@@ -38,20 +173,56 @@ __global__ void __launch_bounds__(kExThreads) exhaustive_kernel(const DockArgs a
   const int n = a.lig.rot_off[l + 1] - r0;   // <= kExMaxRot (checked on the host)
   if (!lg_check(a.grid.check, N <= LIGEN_MAX_ATOMS && n <= kExMaxRot, kChkItemShape)) return;   // uniform
 
-  for (int i = tid; i < N; i += kExThreads) sx[i] = a.pk.xc[a0 + i];
-  for (int w = tid; w < kExMaxRot * (LIGEN_MAX_ATOMS / 32); w += kExThreads) (&member[0][0])[w] = 0u;
+  for (int i = tid; i < N; i += kExThreads) {
+    S.sx[i] = a.pk.xc[a0 + i];
+    S.mask[i] = 0;
+  }
   __syncthreads();
-  for (int b = 0; b < n; ++b) {
+  for (int b = 0; b < n; ++b) {   // one bond after another: a list names an atom once
     const uchar4 bi = a.pk.binfo[r0 + b];
     if (tid == 0) {
-      saxis[b][0] = bi.x;
-      saxis[b][1] = bi.y;
+      S.axis[b][0] = bi.x;
+      S.axis[b][1] = bi.y;
       lg_check(a.grid.check, bi.x < N && bi.y < N, kChkAtomIndex);
     }
     for (int t = tid; t < bi.z; t += kExThreads) {
       const int i = a.pk.frag[(size_t)(r0 + b) * kFragStride + t];
       if (!lg_check(a.grid.check, i < N, kChkAtomIndex)) continue;
-      atomicOr(&member[b][i >> 5], 1u << (i & 31));
+      S.mask[i] |= (uint8_t)(1u << b);
+    }
+    __syncthreads();
+  }
+  // table layout for one rotation: atoms by ascending count of bonds, then by index
+  const unsigned nt = (unsigned)a.n_theta;
+  if (tid < 32) {
+    int used = 0, slots = 0;
+    long long size = 1;
+    for (int m = 0; m <= n; ++m, size *= nt)
+      for (int w = 0; w < N; w += 32) {
+        const int i = w + tid;
+        const bool in = i < N && __popc(S.mask[i < N ? i : 0]) == m;
+        const unsigned all = __ballot_sync(0xffffffffu, in);
+        const int before = __popc(all & ((1u << tid) - 1u));
+        const long long fit = (kExTable - used) / size;
+        if (in) {
+          const bool tabled = before < fit;
+          unsigned st[kExMaxRot] = {0u, 0u, 0u, 0u};
+          if (tabled) {
+            unsigned s = 1u;
+            for (int b = n - 1; b >= 0; --b)
+              if (S.mask[i] >> b & 1u) { st[b] = s; s *= nt; }
+            S.slot[slots + before] = (uint8_t)i;
+          }
+          S.stride[i] = make_uint2(st[0] | st[1] << 16, st[2] | st[3] << 16);
+          S.base[i] = tabled ? (uint16_t)(used + before * size) : kExDirect;
+        }
+        const int kept = (int)(__popc(all) < fit ? __popc(all) : fit);
+        used += (int)(kept * size);
+        slots += kept;
+      }
+    if (tid == 0) {
+      S.entries = used;
+      S.n_slots = slots;
     }
   }
   __syncthreads();
@@ -72,62 +243,85 @@ __global__ void __launch_bounds__(kExThreads) exhaustive_kernel(const DockArgs a
     o[k] = (t - a.origin[k]) * a.inv_h;
   }
 
-  const int nt = a.n_theta;
-  long long per_k = 1;
+  const ExDiv by_nt(nt);
+  unsigned per_k = 1;   // <= 2^27 (checked on the host)
   for (int b = 0; b < n; ++b) per_k *= nt;
-  const long long total = per_k * a.n_rigid;
-
+  const int k_lo = a.n_rigid * rank / kExCluster, k_hi = a.n_rigid * (rank + 1) / kExCluster;
+  const int batch = S.entries ? max(1, kExTable / S.entries) : k_hi - k_lo;   // rotations tabled together
   float best = -INFINITY;
   long long bestc = 0x7fffffffffffffffll;
-  for (long long c = tid; c < total; c += kExThreads) {
-    long long rem = c;
-    int j[kExMaxRot];
-#pragma unroll
-    for (int b = kExMaxRot - 1; b >= 0; --b) {
-      j[b] = 0;
-      if (b < n) { j[b] = (int)(rem % nt); rem /= nt; }
-    }
-    const int k = (int)rem;
-    // axis of each bond after the earlier bonds: its moving end pv and unit direction kd
-    float pv[kExMaxRot][3], kd[kExMaxRot][3], cs[kExMaxRot], sn[kExMaxRot];
-#pragma unroll
-    for (int b = 0; b < kExMaxRot; ++b) {
-      if (b >= n) break;
-      const int iu = saxis[b][0], iv = saxis[b][1];
-      float pu[3] = {sx[iu].x, sx[iu].y, sx[iu].z};
-      float pw[3] = {sx[iv].x, sx[iv].y, sx[iv].z};
-#pragma unroll
-      for (int e = 0; e < kExMaxRot; ++e) {
-        if (e >= b) break;
-        if (member[e][iu >> 5] >> (iu & 31) & 1u) rodrigues_apply(pu, pv[e], kd[e], cs[e], sn[e]);
-        if (member[e][iv >> 5] >> (iv & 31) & 1u) rodrigues_apply(pw, pv[e], kd[e], cs[e], sn[e]);
+  for (int k0 = k_lo; k0 < k_hi; k0 += batch) {
+    const int nk = min(batch, k_hi - k0);
+    for (int e = tid; e < nk * S.entries; e += kExThreads) {
+      const int kk = e / S.entries;
+      unsigned q = (unsigned)(e - kk * S.entries);
+      int lo = 0, hi = S.n_slots - 1;   // last slot that starts at or before q
+      while (lo < hi) {
+        const int mid = (lo + hi + 1) / 2;
+        if (S.base[S.slot[mid]] <= q) lo = mid; else hi = mid - 1;
       }
-      const float d0 = pw[0] - pu[0], d1 = pw[1] - pu[1], d2 = pw[2] - pu[2];
-      const float inv = rsqrtf(d0 * d0 + d1 * d1 + d2 * d2);
-      kd[b][0] = d0 * inv; kd[b][1] = d1 * inv; kd[b][2] = d2 * inv;
-      pv[b][0] = pw[0]; pv[b][1] = pw[1]; pv[b][2] = pw[2];
-      torsion_cs(j[b], a.step_deg, &cs[b], &sn[b]);
-    }
-    float G[9], Mk[9];
-    cube_mat(k, G);
-    mat3mul(M, G, Mk);
-    float acc = 0.f;
-    for (int i = 0; i < N; ++i) {
-      const float4 X = sx[i];
-      float y[3] = {X.x, X.y, X.z};
+      const int i = S.slot[lo];
+      const unsigned mask = S.mask[i];
+      q -= S.base[i];
+      int j[kExMaxRot];
 #pragma unroll
-      for (int b = 0; b < kExMaxRot; ++b) {
-        if (b >= n) break;
-        if (member[b][i >> 5] >> (i & 31) & 1u) rodrigues_apply(y, pv[b], kd[b], cs[b], sn[b]);
+      for (int b = kExMaxRot - 1; b >= 0; --b) {
+        j[b] = 0;
+        if (mask >> b & 1u) {
+          const unsigned up = by_nt(q);
+          j[b] = (int)(q - up * nt);
+          q = up;
+        }
       }
-      const float ux = fmaf(Mk[0], y[0], fmaf(Mk[1], y[1], fmaf(Mk[2], y[2], o[0])));
-      const float uy = fmaf(Mk[3], y[0], fmaf(Mk[4], y[1], fmaf(Mk[5], y[2], o[1])));
-      const float uz = fmaf(Mk[6], y[0], fmaf(Mk[7], y[1], fmaf(Mk[8], y[2], o[2])));
-      acc -= grid_sample_fmt<FMT>(a.grid, ux, uy, uz, __float_as_int(X.w));
+      float pv[kExMaxRot][3], kd[kExMaxRot][3], cs[kExMaxRot], sn[kExMaxRot];
+      ex_axes(S, mask, n, j, a.step_deg, pv, kd, cs, sn);
+      float G[9], Mk[9];
+      cube_mat(k0 + kk, G);
+      mat3mul(M, G, Mk);
+      tab[e] = ex_energy<FMT>(a, S, i, n, Mk, o, pv, kd, cs, sn);
     }
-    if (acc > best) { best = acc; bestc = c; }   // c ascends per thread: ties keep the first
+    __syncthreads();
+    const unsigned total = per_k * (unsigned)nk;
+    const long long c0 = (long long)k0 * per_k;
+    if (S.n_slots == N) {
+      if (n <= 1) ex_sum<1>(S, tab, N, n, by_nt, total, c0, best, bestc);
+      else if (n == 2) ex_sum<2>(S, tab, N, n, by_nt, total, c0, best, bestc);
+      else if (n == 3) ex_sum<3>(S, tab, N, n, by_nt, total, c0, best, bestc);
+      else ex_sum<4>(S, tab, N, n, by_nt, total, c0, best, bestc);
+    } else {
+      for (unsigned t = tid; t < total; t += kExThreads) {
+        unsigned q = t;
+        int j[kExMaxRot];
+#pragma unroll
+        for (int b = kExMaxRot - 1; b >= 0; --b) {
+          j[b] = 0;
+          if (b < n) {
+            const unsigned up = by_nt(q);
+            j[b] = (int)(q - up * nt);
+            q = up;
+          }
+        }
+        float pv[kExMaxRot][3], kd[kExMaxRot][3], cs[kExMaxRot], sn[kExMaxRot];
+        ex_axes(S, 0xfu, n, j, a.step_deg, pv, kd, cs, sn);
+        float G[9], Mk[9];
+        cube_mat(k0 + (int)q, G);
+        mat3mul(M, G, Mk);
+        float acc = 0.f;
+        for (int i = 0; i < N; ++i) {
+          if (S.base[i] != kExDirect) {   // uniform
+            const uint2 s = S.stride[i];
+            acc -= tab[S.base[i] + q * S.entries + j[0] * (s.x & 0xffffu) + j[1] * (s.x >> 16) +
+                       j[2] * (s.y & 0xffffu) + j[3] * (s.y >> 16)];
+          } else {
+            acc -= ex_energy<FMT>(a, S, i, n, Mk, o, pv, kd, cs, sn);
+          }
+        }
+        if (acc > best) { best = acc; bestc = c0 + t; }   // t ascends per thread: ties keep the first
+      }
+    }
+    __syncthreads();
   }
-  // block argmax: higher score, then lower combination index
+  // argmax: higher score, then lower combination index
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) {
     const float os = __shfl_xor_sync(0xffffffffu, best, off);
@@ -139,29 +333,44 @@ __global__ void __launch_bounds__(kExThreads) exhaustive_kernel(const DockArgs a
   if (tid == 0) {
     for (int w = 1; w < kExThreads / 32; ++w)
       if (red_s[w] > best || (red_s[w] == best && red_c[w] < bestc)) { best = red_s[w]; bestc = red_c[w]; }
+    cta_s = best;
+    cta_c = bestc;
+  }
+  cg::cluster_group cluster = cg::this_cluster();
+  cluster.sync();
+  if (rank == 0 && tid == 0) {
+    for (int c = 1; c < kExCluster; ++c) {
+      const float os = *cluster.map_shared_rank(&cta_s, c);
+      const long long oc = *cluster.map_shared_rank(&cta_c, c);
+      if (os > best || (os == best && oc < bestc)) { best = os; bestc = oc; }
+    }
+    const long long total = (long long)per_k * a.n_rigid;
     if (bestc >= total) bestc = 0;   // only if every score is NaN; keeps the indices in range
     const size_t lr = (size_t)l * a.R + r;
-    if (a.samples) atomicAdd(&a.samples[blockIdx.x % kSampleSlots], (unsigned long long)(total * N));
+    if (a.samples) atomicAdd(&a.samples[item % kSampleSlots], (unsigned long long)(total * N));
     a.res_score[lr] = best;
     long long rem = bestc;
     uint8_t* cnt = a.res_cnt + (size_t)r0 * a.R + (size_t)r * n;
     for (int b = n - 1; b >= 0; --b) { cnt[b] = (uint8_t)(rem % nt); rem /= nt; }
     a.res_k[lr] = (uint8_t)rem;
   }
+  cluster.sync();   // the other CTAs' winners stay readable until here
 }
 
 }  // namespace
 
 cudaError_t launch_exhaustive(const DockArgs& a, cudaStream_t s) {
-  const long long blocks = (long long)a.lig.L * a.R;
-  if (blocks == 0) return cudaSuccess;
-  if (a.fmt == kRecF32)
-    exhaustive_kernel<kRecF32><<<(unsigned)blocks, kExThreads, 0, s>>>(a);
-  else if (a.fmt == kRecF16)
-    exhaustive_kernel<kRecF16><<<(unsigned)blocks, kExThreads, 0, s>>>(a);
-  else
-    exhaustive_kernel<kRecBF16><<<(unsigned)blocks, kExThreads, 0, s>>>(a);
-  return cudaGetLastError();
+  const auto kernel = a.fmt == kRecF32   ? exhaustive_kernel<kRecF32>
+                      : a.fmt == kRecF16 ? exhaustive_kernel<kRecF16>
+                                         : exhaustive_kernel<kRecBF16>;
+  const long long items = (long long)a.lig.L * a.R, most = (1ll << 31) / kExCluster - 1;   // grid limit
+  for (long long first = 0; first < items; first += most) {
+    const long long here = items - first < most ? items - first : most;
+    kernel<<<(unsigned)(here * kExCluster), kExThreads, 0, s>>>(a, first);
+    const cudaError_t e = cudaGetLastError();
+    if (e != cudaSuccess) return e;
+  }
+  return cudaSuccess;
 }
 
 }  // namespace ligen
