@@ -134,8 +134,10 @@ typedef struct ligen_grid {
 
 /* How the docking work of a call is laid out on the GPU (same results).
  *   LIGEN_BATCH_PLAIN    one launch over the library, one CTA per (ligand,
- *                        restart chunk), shared memory sized for the largest
- *                        ligand of the call;
+ *                        restart chunk), the ligands with the most estimated
+ *                        work first, shared memory sized for the largest
+ *                        ligand of the call; 8 lanes per restart, or 16 or 32
+ *                        when the call is too small to fill the device;
  *   LIGEN_BATCH_BUCKETS  paper §3: ligands are grouped by atom class x
  *                        rotamer class (the bucket ids of ligen_pack_ligands)
  *                        and ordered largest-cost first; each atom class runs

@@ -166,7 +166,13 @@ cudaError_t launch_grid_prep_fmt(const float* values, int nx, int ny, int nz, in
 // max_atoms: the library's largest ligand. With out.fk_xs set, the
 // forward-kinematics table (out.fk_*) too.
 cudaError_t launch_pack(const LigandsDev& lig, int nc, const Packed& out, int max_atoms, cudaStream_t s);
+// The ligands by decreasing estimated docking cost (order [L]).
+cudaError_t launch_order(const LigandsDev& lig, int n_rigid, int passes, int n_theta, int32_t* order,
+                         cudaStream_t s);
 size_t dock_smem_bytes(int max_atoms, int max_rot, int max_frag, int rpc);
+// Lanes per restart for a plain launch of this library and search.
+int dock_pick_lanes(const int32_t* h_atom_off, const int32_t* h_rot_off, int L, int R, int n_rigid, int n_theta,
+                    int passes, int fmt, int sms);
 bool dock_lanes_supported(int lanes);
 bool dock_shape_supported(int lanes, int fmt);
 // grid_ctas: CTAs of a persistent launch (ignored when a.queue is NULL).

@@ -8,7 +8,10 @@
 // increments in the sweep) and each lane sums its candidates' atom terms on
 // its own, so a stage needs no per-candidate reduction, only a log2(G)-step
 // shuffle argmax across the group. A lane holds SLOTS increments, so SLOTS
-// independent 256-bit gathers are in flight per moving atom.
+// independent 256-bit gathers are in flight per moving atom; the wide shapes
+// (a restart per half-warp or warp, for launches too small to fill the chip)
+// also take UT moving atoms at once, since there the chain of loads is the
+// time. Every shape adds in the same order, so results do not depend on it.
 //
 // Shared memory per CTA: the ligand (centred coordinates + type, bond axes,
 // moving-atom lists) and the current coordinates of every restart, in grid
@@ -21,6 +24,9 @@
 // persistent grid whose CTAs take items from a device counter (atomicAdd,
 // no waiting) until the list is exhausted; items may come from a ligand list
 // (a bucket of similar ligands) instead of the whole library.
+#include <algorithm>
+#include <cmath>
+
 #include "../../include/ligen.h"
 #include "internal.h"
 
@@ -87,7 +93,7 @@ __device__ __forceinline__ void group_argmax(float& s, int& idx) {
 // One work item: ligand l, restarts [chunk * rpc, chunk * rpc + rpc).
 // COUNT: also add the samples the item's restarts needed to a.samples (a
 // separate instantiation, so the plain kernel carries no counting).
-template <int G, int SLOTS, int FMT, bool COUNT>
+template <int G, int SLOTS, int FMT, bool COUNT, int UT>
 __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S, int l, int chunk) {
   const int rpc = a.rpc;
   const int tid = threadIdx.x;
@@ -150,6 +156,7 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
     o[k] = (t - a.origin[k]) * a.inv_h;
   }
 
+  constexpr int kRigidUnroll = UT > 1 ? 8 : 4;
   // ---- rigid stage: lane `sub` scores cube rotations sub, sub+G, ...
   float best = -INFINITY;
   int kb = 0;
@@ -158,14 +165,15 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
     cube_mat(k, Gk);
     mat3mul(M, Gk, Mk);
     float acc = 0.f;
-#pragma unroll 4
+#pragma unroll kRigidUnroll
     for (int i = 0; i < N; ++i) {
       const float4 X = S.sx[i];
       const float ux = fmaf(Mk[0], X.x, fmaf(Mk[1], X.y, fmaf(Mk[2], X.z, o[0])));
       const float uy = fmaf(Mk[3], X.x, fmaf(Mk[4], X.y, fmaf(Mk[5], X.z, o[1])));
       const float uz = fmaf(Mk[6], X.x, fmaf(Mk[7], X.y, fmaf(Mk[8], X.z, o[2])));
       const int c = __float_as_int(X.w);
-      if constexpr (FMT == kRecF32) acc -= grid_sample(grid, ux, uy, uz, c);
+      if constexpr (UT > 1) acc -= grid_sample_nb_fmt<FMT>(grid, ux, uy, uz, c);
+      else if constexpr (FMT == kRecF32) acc -= grid_sample(grid, ux, uy, uz, c);
       else acc -= grid_sample16_cb<FMT>(grid, chan_base16(grid, c), ux, uy, uz, c);
     }
     if (acc > best) { best = acc; kb = k; }
@@ -248,43 +256,75 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
         // keeps j = 0, the decision a sweep would reach.
         const int m_live = live ? m : 0;
         if (COUNT && ch == 0) needed += (long long)(nt - 1) * m_live;
-        for (int t = 0; t < m_live; ++t) {
-          const int i = S.sfrag[off + t];
-          const int c = __float_as_int(S.sx[i].w);
-          const unsigned char* cb = FMT == kRecF32 ? nullptr : chan_base16(grid, c);   // 16-bit records
-          const float dx = S.cx[i * rpc + rr] - vx;
-          const float dy = S.cy[i * rpc + rr] - vy;
-          const float dz = S.cz[i * rpc + rr] - vz;
-          const float kd = kx * dx + ky * dy + kz * dz;
-          const float px = fmaf(kx, kd, vx), py = fmaf(ky, kd, vy), pz = fmaf(kz, kd, vz);
-          const float ex = fmaf(-kx, kd, dx), ey = fmaf(-ky, kd, dy), ez = fmaf(-kz, kd, dz);
-          const float qx = ky * dz - kz * dy, qy = kz * dx - kx * dz, qz = kx * dy - ky * dx;
-          if constexpr (FMT != kRecF32) {
-            // two increments per packed instruction (measured: 0.5% faster
-            // with 16-bit records, 1% slower with FP32 records)
-            float ux[SLOTS], uy[SLOTS], uz[SLOTS];
+        if constexpr (UT > 1) {
+          // UT atoms' samples in flight, added in list order
+          for (int t0 = 0; t0 < m_live; t0 += UT) {
+            float e[UT][SLOTS];
 #pragma unroll
-            for (int s = 0; s + 1 < SLOTS; s += 2) {
-              const float2 cc = make_float2(cs[s], cs[s + 1]), ss = make_float2(sn[s], sn[s + 1]);
-              const float2 X = fma2(make_float2(ex, ex), cc, fma2(make_float2(qx, qx), ss, make_float2(px, px)));
-              const float2 Y = fma2(make_float2(ey, ey), cc, fma2(make_float2(qy, qy), ss, make_float2(py, py)));
-              const float2 Z = fma2(make_float2(ez, ez), cc, fma2(make_float2(qz, qz), ss, make_float2(pz, pz)));
-              ux[s] = X.x; ux[s + 1] = X.y; uy[s] = Y.x; uy[s + 1] = Y.y; uz[s] = Z.x; uz[s + 1] = Z.y;
-            }
-            if constexpr (SLOTS % 2 == 1) {
-              ux[SLOTS - 1] = fmaf(ex, cs[SLOTS - 1], fmaf(qx, sn[SLOTS - 1], px));
-              uy[SLOTS - 1] = fmaf(ey, cs[SLOTS - 1], fmaf(qy, sn[SLOTS - 1], py));
-              uz[SLOTS - 1] = fmaf(ez, cs[SLOTS - 1], fmaf(qz, sn[SLOTS - 1], pz));
+            for (int q = 0; q < UT; ++q) {
+              const int i = S.sfrag[off + min(t0 + q, m_live - 1)];   // past the end: the last atom again, not added
+              const int c = __float_as_int(S.sx[i].w);
+              const float dx = S.cx[i * rpc + rr] - vx;
+              const float dy = S.cy[i * rpc + rr] - vy;
+              const float dz = S.cz[i * rpc + rr] - vz;
+              const float kd = kx * dx + ky * dy + kz * dz;
+              const float px = fmaf(kx, kd, vx), py = fmaf(ky, kd, vy), pz = fmaf(kz, kd, vz);
+              const float ex = fmaf(-kx, kd, dx), ey = fmaf(-ky, kd, dy), ez = fmaf(-kz, kd, dz);
+              const float qx = ky * dz - kz * dy, qy = kz * dx - kx * dz, qz = kx * dy - ky * dx;
+#pragma unroll
+              for (int s = 0; s < SLOTS; ++s) {
+                const float ux = fmaf(ex, cs[s], fmaf(qx, sn[s], px));
+                const float uy = fmaf(ey, cs[s], fmaf(qy, sn[s], py));
+                const float uz = fmaf(ez, cs[s], fmaf(qz, sn[s], pz));
+                e[q][s] = grid_sample_nb_fmt<FMT>(grid, ux, uy, uz, c);
+              }
             }
 #pragma unroll
-            for (int s = 0; s < SLOTS; ++s) acc[s] -= grid_sample16_cb<FMT>(grid, cb, ux[s], uy[s], uz[s], c);
-          } else {
+            for (int q = 0; q < UT; ++q)
+              if (t0 + q < m_live) {
 #pragma unroll
-            for (int s = 0; s < SLOTS; ++s) {
-              const float ux = fmaf(ex, cs[s], fmaf(qx, sn[s], px));
-              const float uy = fmaf(ey, cs[s], fmaf(qy, sn[s], py));
-              const float uz = fmaf(ez, cs[s], fmaf(qz, sn[s], pz));
-              acc[s] -= grid_sample_fmt<FMT>(grid, ux, uy, uz, c);
+                for (int s = 0; s < SLOTS; ++s) acc[s] -= e[q][s];
+              }
+          }
+        } else {
+          for (int t = 0; t < m_live; ++t) {
+            const int i = S.sfrag[off + t];
+            const int c = __float_as_int(S.sx[i].w);
+            const unsigned char* cb = FMT == kRecF32 ? nullptr : chan_base16(grid, c);   // 16-bit records
+            const float dx = S.cx[i * rpc + rr] - vx;
+            const float dy = S.cy[i * rpc + rr] - vy;
+            const float dz = S.cz[i * rpc + rr] - vz;
+            const float kd = kx * dx + ky * dy + kz * dz;
+            const float px = fmaf(kx, kd, vx), py = fmaf(ky, kd, vy), pz = fmaf(kz, kd, vz);
+            const float ex = fmaf(-kx, kd, dx), ey = fmaf(-ky, kd, dy), ez = fmaf(-kz, kd, dz);
+            const float qx = ky * dz - kz * dy, qy = kz * dx - kx * dz, qz = kx * dy - ky * dx;
+            if constexpr (FMT != kRecF32) {
+              // two increments per packed instruction (measured: 0.5% faster
+              // with 16-bit records, 1% slower with FP32 records)
+              float ux[SLOTS], uy[SLOTS], uz[SLOTS];
+#pragma unroll
+              for (int s = 0; s + 1 < SLOTS; s += 2) {
+                const float2 cc = make_float2(cs[s], cs[s + 1]), ss = make_float2(sn[s], sn[s + 1]);
+                const float2 X = fma2(make_float2(ex, ex), cc, fma2(make_float2(qx, qx), ss, make_float2(px, px)));
+                const float2 Y = fma2(make_float2(ey, ey), cc, fma2(make_float2(qy, qy), ss, make_float2(py, py)));
+                const float2 Z = fma2(make_float2(ez, ez), cc, fma2(make_float2(qz, qz), ss, make_float2(pz, pz)));
+                ux[s] = X.x; ux[s + 1] = X.y; uy[s] = Y.x; uy[s + 1] = Y.y; uz[s] = Z.x; uz[s + 1] = Z.y;
+              }
+              if constexpr (SLOTS % 2 == 1) {
+                ux[SLOTS - 1] = fmaf(ex, cs[SLOTS - 1], fmaf(qx, sn[SLOTS - 1], px));
+                uy[SLOTS - 1] = fmaf(ey, cs[SLOTS - 1], fmaf(qy, sn[SLOTS - 1], py));
+                uz[SLOTS - 1] = fmaf(ez, cs[SLOTS - 1], fmaf(qz, sn[SLOTS - 1], pz));
+              }
+#pragma unroll
+              for (int s = 0; s < SLOTS; ++s) acc[s] -= grid_sample16_cb<FMT>(grid, cb, ux[s], uy[s], uz[s], c);
+            } else {
+#pragma unroll
+              for (int s = 0; s < SLOTS; ++s) {
+                const float ux = fmaf(ex, cs[s], fmaf(qx, sn[s], px));
+                const float uy = fmaf(ey, cs[s], fmaf(qy, sn[s], py));
+                const float uz = fmaf(ez, cs[s], fmaf(qz, sn[s], pz));
+                acc[s] -= grid_sample_fmt<FMT>(grid, ux, uy, uz, c);
+              }
             }
           }
         }
@@ -326,13 +366,22 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
     }
   }
 
-  // ---- final score of the restart's pose (all atoms)
+  // ---- final score of the restart's pose (all atoms), in at most 8 partial
+  // sums whatever the group's width (wider groups repeat them: same loads)
+  constexpr int FG = G < 8 ? G : 8;
   float acc = 0.f;
-  for (int i = sub; i < N; i += G)
-    acc -= grid_sample_fmt<FMT>(grid, S.cx[i * rpc + rr], S.cy[i * rpc + rr], S.cz[i * rpc + rr],
-                       __float_as_int(S.sx[i].w));
+  if constexpr (UT > 1) {
+#pragma unroll 4
+    for (int i = sub % FG; i < N; i += FG)
+      acc -= grid_sample_nb_fmt<FMT>(grid, S.cx[i * rpc + rr], S.cy[i * rpc + rr], S.cz[i * rpc + rr],
+                                     __float_as_int(S.sx[i].w));
+  } else {
+    for (int i = sub; i < N; i += G)
+      acc -= grid_sample_fmt<FMT>(grid, S.cx[i * rpc + rr], S.cy[i * rpc + rr], S.cz[i * rpc + rr],
+                                  __float_as_int(S.sx[i].w));
+  }
 #pragma unroll
-  for (int off = 1; off < G; off <<= 1) acc += __shfl_xor_sync(kFull, acc, off);
+  for (int off = 1; off < FG; off <<= 1) acc += __shfl_xor_sync(kFull, acc, off);
   if constexpr (COUNT) {   // one add per warp, spread over the counter slots
     long long v = (active && sub == 0) ? needed : 0;
 #pragma unroll
@@ -365,7 +414,7 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
 // 7 (8 leave under 48 KB of L1 and run 60% slower; 6 CTAs 9%, the
 // unconstrained build 42%).
 // launch_dock takes the largest count whose CTAs fit kCtaSmemBudget.
-template <int G, int SLOTS, int FMT, bool COUNT, int MINB>
+template <int G, int SLOTS, int FMT, bool COUNT, int MINB, int UT>
 __global__ void __launch_bounds__(128, MINB) dock_kernel(const DockArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int next_item;
@@ -383,7 +432,7 @@ __global__ void __launch_bounds__(128, MINB) dock_kernel(const DockArgs a) {
     const int li = item / a.chunks;
     const int l = a.list ? a.list[li] : li;
     if (a.pk.status[l] == 0)   // uniform over the CTA
-      dock_item<G, SLOTS, FMT, COUNT>(a, S, l, item - li * a.chunks);
+      dock_item<G, SLOTS, FMT, COUNT, UT>(a, S, l, item - li * a.chunks);
     if (!a.queue) break;
     __syncthreads();   // shared memory is reused by the next item
   }
@@ -400,42 +449,60 @@ namespace {
 using KernelFn = void (*)(DockArgs);
 
 
+// Resident CTAs asked of the register allocator: `ctas` for the 8-lane
+// shapes (see dock_kernel); 4 for the 16-lane ones (128 registers) and 3 for
+// the 32-lane ones (168). Left to itself the allocator takes 200-254 for the
+// gathers in flight, two CTAs per SM: that is 15-20% faster while one CTA
+// per SM runs (5 screening ligands 92 against 111 us with four) and 20-30%
+// slower from a few dozen ligands on (160 ligands on 16 lanes 731 against
+// 553 us).
+constexpr int build_ctas(int G, int ctas) { return G == 8 ? ctas : G == 16 ? 4 : G == 32 ? 3 : 1; }
+
 // Instantiated (G, SLOTS, record format) shapes; G * SLOTS increments per
-// chunk of the sweep. The 16-bit record formats exist for 4 and 8 lanes.
+// chunk of the sweep.
 struct Shape {
   int G, SLOTS, FMT;
   KernelFn fn[2][4];   // [counts the samples needed][build: 8, 7, 6 CTAs, unconstrained]
 };
-#define LG_BUILDS(G, S, F, C)                                                                         \
-  {dock_kernel<G, S, F, C, G == 8 ? 8 : 1>, dock_kernel<G, S, F, C, G == 8 ? 7 : 1>,                   \
-   dock_kernel<G, S, F, C, G == 8 ? 6 : 1>, dock_kernel<G, S, F, C, 1>}
+#define LG_BUILDS(G, S, F, C, U)                                                                      \
+  {dock_kernel<G, S, F, C, build_ctas(G, 8), U>, dock_kernel<G, S, F, C, build_ctas(G, 7), U>,         \
+   dock_kernel<G, S, F, C, build_ctas(G, 6), U>, dock_kernel<G, S, F, C, build_ctas(G, 1), U>}
 // The counting kernel only serves untimed calls: one build for all four.
-#define LG_COUNTING(G, S, F)                                                                          \
-  {dock_kernel<G, S, F, true, 1>, dock_kernel<G, S, F, true, 1>, dock_kernel<G, S, F, true, 1>,        \
-   dock_kernel<G, S, F, true, 1>}
-#define LG_SHAPE(G, S, F) {G, S, F, {LG_BUILDS(G, S, F, false), LG_COUNTING(G, S, F)}}
+#define LG_COUNTING(G, S, F, U)                                                                          \
+  {dock_kernel<G, S, F, true, 1, U>, dock_kernel<G, S, F, true, 1, U>, dock_kernel<G, S, F, true, 1, U>,  \
+   dock_kernel<G, S, F, true, 1, U>}
+#define LG_SHAPE(G, S, F, U) {G, S, F, {LG_BUILDS(G, S, F, false, U), LG_COUNTING(G, S, F, U)}}
 const Shape kShapes[] = {
-    LG_SHAPE(2, 6, kRecF32),
-    LG_SHAPE(2, 18, kRecF32),
-    LG_SHAPE(4, 3, kRecF32),
-    LG_SHAPE(4, 9, kRecF32),
-    LG_SHAPE(8, 2, kRecF32),
-    LG_SHAPE(8, 5, kRecF32),
-    LG_SHAPE(4, 3, kRecF16),
-    LG_SHAPE(4, 9, kRecF16),
-    LG_SHAPE(8, 2, kRecF16),
-    LG_SHAPE(8, 5, kRecF16),
-    LG_SHAPE(4, 3, kRecBF16),
-    LG_SHAPE(4, 9, kRecBF16),
-    LG_SHAPE(8, 2, kRecBF16),
-    LG_SHAPE(8, 5, kRecBF16),
+    LG_SHAPE(2, 6, kRecF32, 1),
+    LG_SHAPE(2, 18, kRecF32, 1),
+    LG_SHAPE(4, 3, kRecF32, 1),
+    LG_SHAPE(4, 9, kRecF32, 1),
+    LG_SHAPE(8, 2, kRecF32, 1),
+    LG_SHAPE(8, 5, kRecF32, 1),
+    LG_SHAPE(4, 3, kRecF16, 1),
+    LG_SHAPE(4, 9, kRecF16, 1),
+    LG_SHAPE(8, 2, kRecF16, 1),
+    LG_SHAPE(8, 5, kRecF16, 1),
+    LG_SHAPE(4, 3, kRecBF16, 1),
+    LG_SHAPE(4, 9, kRecBF16, 1),
+    LG_SHAPE(8, 2, kRecBF16, 1),
+    LG_SHAPE(8, 5, kRecBF16, 1),
     // one restart per half-warp or warp: a gather request covers 16 or 32
     // consecutive increments of one atom of one restart (36 increments as
-    // 3 x 16 or 2 x 32 slots, the spare lanes repeating a valid increment)
-    LG_SHAPE(16, 3, kRecF32),
-    LG_SHAPE(32, 2, kRecF32),
-    LG_SHAPE(16, 3, kRecF16),
-    LG_SHAPE(32, 2, kRecF16),
+    // 3 x 16 or 2 x 32 slots, the spare lanes repeating a valid increment),
+    // SLOTS * UT gathers in flight
+    LG_SHAPE(16, 1, kRecF32, 4),
+    LG_SHAPE(16, 3, kRecF32, 2),
+    LG_SHAPE(32, 1, kRecF32, 4),
+    LG_SHAPE(32, 2, kRecF32, 4),
+    LG_SHAPE(16, 1, kRecF16, 4),
+    LG_SHAPE(16, 3, kRecF16, 2),
+    LG_SHAPE(32, 1, kRecF16, 4),
+    LG_SHAPE(32, 2, kRecF16, 4),
+    LG_SHAPE(16, 1, kRecBF16, 4),
+    LG_SHAPE(16, 3, kRecBF16, 2),
+    LG_SHAPE(32, 1, kRecBF16, 4),
+    LG_SHAPE(32, 2, kRecBF16, 4),
 };
 #undef LG_SHAPE
 #undef LG_COUNTING
@@ -469,7 +536,63 @@ const Shape* pick_shape(int G, int n_theta, int fmt) {
   return best;
 }
 
+// Sweep slots a group computes per moving atom: n_theta rounded up to whole
+// lanes and chunks.
+int sweep_slots(int G, int n_theta, int fmt) {
+  const Shape* sh = pick_shape(G, n_theta, fmt);
+  const int per = sh->G * sh->SLOTS;
+  return (n_theta + per - 1) / per * per;
+}
+
 }  // namespace
+
+// Lanes per restart of a plain launch. A launch that fills the chip is
+// fastest with 8 (each sample costs the same whatever the lanes, and fewer
+// instructions are spent on spare lanes); one that does not lasts as long as
+// the chain of loads of its largest ligand, which 16 or 32 lanes shorten. The
+// time is estimated for each as hypot(largest ligand's chain, total work /
+// rate) and the shortest taken. Work counts the candidate samples of the
+// rigid stage and of full sweeps of n_theta = 36 slots, (N + 4) / 4 moving
+// atoms a bond (plan_groups' estimate) and a constant per restart for the
+// rest. Constants fitted to launches of 1-20,000 screening, 1-5,000 bimodal
+// and 32-3,000 small ligands on GB300, longest ligand first; measured
+// docking kernel (us), chosen one first:
+//                        5 ligands   20        80        160       320
+//   screening   8 lanes  430         311       354       621       817*
+//              16 lanes  145         125       279*      553*      1454
+//              32 lanes  92*         115*      397       797       2123
+//   bimodal     8 lanes  788         866       1032      1202      1325*
+//              16 lanes  256         309       434*      850*      1632
+//              32 lanes  164*        242*      590       1196      2312
+int dock_pick_lanes(const int32_t* h_atom_off, const int32_t* h_rot_off, int L, int R, int n_rigid, int n_theta,
+                    int passes, int fmt, int sms) {
+  struct Model {
+    int lanes;
+    double us, us_per_cost, cost_per_us;   // chain: us + us_per_cost * cost; throughput
+  };
+  constexpr Model kModels[] = {{8, 50., 0.0135, 1.143e6}, {16, 40., 0.0036, 0.766e6}, {32, 40., 0.0024, 0.522e6}};
+  constexpr double kRestart = 2000.;   // cost of a restart outside its samples
+  constexpr int kSms = 152;            // of the measurements
+  if ((double)L * R > 400. * sms) return 8;   // fills the chip with any ligands
+  int best = 8;
+  double best_us = 0.;
+  for (const Model& m : kModels) {
+    const double slots = 36. * sweep_slots(m.lanes, n_theta, fmt) / sweep_slots(m.lanes, 36, fmt);
+    double work = 0., largest = 0.;
+    for (int l = 0; l < L; ++l) {
+      const double N = h_atom_off[l + 1] - h_atom_off[l], n = h_rot_off[l + 1] - h_rot_off[l];
+      const double rigid = n_rigid * N, moving = passes * n * (N + 4.) / 4.;
+      work += rigid + slots * moving + kRestart;
+      largest = std::max(largest, rigid + 36. * moving);
+    }
+    const double us = std::hypot(m.us + m.us_per_cost * largest, work * R / (m.cost_per_us * sms / kSms));
+    if (m.lanes == 8 || us < best_us) {
+      best = m.lanes;
+      best_us = us;
+    }
+  }
+  return best;
+}
 
 bool dock_lanes_supported(int G) { return G == 2 || G == 4 || G == 8 || G == 16 || G == 32; }
 

@@ -413,7 +413,53 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(const LigandsDev 
   }
 }
 
+// Ligands by decreasing estimated docking cost (the cost of plan_groups):
+// one CTA, a counting sort over the cost's exponent and three mantissa bits,
+// so ligands within 1/8 of each other come in any order.
+constexpr int kOrderThreads = 1024;
+constexpr int kOrderBins = 512;
+
+__global__ void __launch_bounds__(kOrderThreads) order_kernel(const LigandsDev lig, int n_rigid, int passes,
+                                                              int n_theta, int32_t* order) {
+  __shared__ int start[kOrderBins];
+  __shared__ int warp_sum[kOrderBins / 32];
+  const int tid = threadIdx.x;
+  auto bin = [&](int l) {
+    const int N = lig.atom_off[l + 1] - lig.atom_off[l], n = lig.rot_off[l + 1] - lig.rot_off[l];
+    const float c = 4.f * N * n_rigid + (float)passes * n * n_theta * (N + 4);
+    const int b = (int)(__float_as_uint(c) >> 20) - (127 << 3);   // c >= 1: 8 bins per power of two
+    return kOrderBins - 1 - min(max(b, 0), kOrderBins - 1);
+  };
+  if (tid < kOrderBins) start[tid] = 0;
+  __syncthreads();
+  for (int l = tid; l < lig.L; l += kOrderThreads) atomicAdd(&start[bin(l)], 1);
+  __syncthreads();
+  int v = 0, sum = 0;   // exclusive prefix sums
+  if (tid < kOrderBins) {
+    v = sum = start[tid];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int t = __shfl_up_sync(kFull, sum, o);
+      if ((tid & 31) >= o) sum += t;
+    }
+    if ((tid & 31) == 31) warp_sum[tid >> 5] = sum;
+  }
+  __syncthreads();
+  if (tid < kOrderBins) {
+    for (int w = 0; w < tid >> 5; ++w) sum += warp_sum[w];
+    start[tid] = sum - v;
+  }
+  __syncthreads();
+  for (int l = tid; l < lig.L; l += kOrderThreads) order[atomicAdd(&start[bin(l)], 1)] = l;
+}
+
 }  // namespace
+
+cudaError_t launch_order(const LigandsDev& lig, int n_rigid, int passes, int n_theta, int32_t* order,
+                         cudaStream_t s) {
+  order_kernel<<<1, kOrderThreads, 0, s>>>(lig, n_rigid, passes, n_theta, order);
+  return cudaGetLastError();
+}
 
 cudaError_t launch_pack(const LigandsDev& lig, int nc, const Packed& out, int max_atoms, cudaStream_t s) {
   if (lig.L == 0) return cudaSuccess;
