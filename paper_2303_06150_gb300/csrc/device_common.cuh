@@ -147,6 +147,11 @@ struct GridView {
   int cx, cy, cz;      // record cells per axis (rec_cells of the format)
   int nc;
   float mx, my, mz;    // points - 1 per axis, as float: upper box bound in grid units
+  // operands of the docking kernel's sampler (DockPoint)
+  float lx, ly, lz;    // the floats below mx, my, mz
+  unsigned hx, hy, hz; // bits of mx, my, mz
+  unsigned cells;      // cx cy cz, modulo 2^32
+  unsigned bias;       // the bits of 2^23 times (cy cx + cx + 1), modulo 2^32
   float penalty;
   size_t n_rec;        // records in the buffer (checked builds compare with it)
   unsigned* check;     // checked builds: first out-of-range code, else NULL
@@ -205,6 +210,12 @@ __device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c) {   // a * 
 __device__ __forceinline__ float2 sub2(float2 a, float2 b) {   // a - b
   unsigned long long d;
   asm("sub.rn.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pk2(a.x, a.y)), "l"(pk2(b.x, b.y)));
+  return upk2(d);
+}
+
+__device__ __forceinline__ float2 add2_rz(float2 a, float2 b) {   // a + b, rounded towards zero
+  unsigned long long d;
+  asm("add.rz.f32x2 %0, %1, %2;" : "=l"(d) : "l"(pk2(a.x, a.y)), "l"(pk2(b.x, b.y)));
   return upk2(d);
 }
 
@@ -356,54 +367,107 @@ __device__ __forceinline__ float grid_sample_fmt(const GridView& g, float ux, fl
   }
 }
 
-// grid_sample_nb for any record format: grid_sample_fmt's value, bit for
-// bit, without a branch around the load.
+// The docking kernel's sampler, in steps, so that two samples share their
+// packed instructions (positions, cells and fractions of a pair). Same values
+// as grid_sample_fmt, bit for bit.
+//
+//   floor     u + 2^23 rounded towards zero has floor(u) in its low mantissa
+//             bits (0 <= u < 2^23) and gives it back as a float by
+//             subtracting 2^23: two full-rate additions instead of a
+//             round-down and a conversion;
+//   clamp     coefficient records end below the upper faces (rec_cells): the
+//             coordinate is cut to the float below n - 1 before its floor, so
+//             a point on a face takes the last cell at f = 1;
+//   inside    the bits of a float order like unsigned integers, negative ones
+//             and NaN above every coordinate of the box: one comparison per
+//             axis. A coordinate of -0 would count as outside; positions here
+//             are sums that start from t - origin, which is never -0;
+//   record    32-bit index arithmetic on the unreduced bits, their constant
+//             part subtracted once (GridView::bias). Bounds, bias and cell
+//             counts are constant-bank operands: none takes a register.
+//
+// Measured on GB300 against floorf, conversions, six comparisons and a clamp
+// per scalar sample (docking kernel, 12,000 screening / 3,000 bimodal
+// ligands): FP32 26.28 -> 23.00 / 11.93 -> 9.59 ms (2,000 screening ligands:
+// 3.67 -> 2.44 G warp instructions, 4.69 -> 3.88 ms, 303 G samples/s of the
+// 308 G/s gather ceiling), FP16 26.25 -> 25.26 / 11.76 -> 11.22 ms.
+constexpr float kFloorMagic = 8388608.f;   // 2^23
+
+struct DockPoint {   // a position, its cell as unreduced bits, its fractions
+  float ux, uy, uz;
+  unsigned bx, by, bz;
+  float dx, dy, dz;
+};
+
 template <int FMT>
-__device__ __forceinline__ float grid_sample_nb_fmt(const GridView& g, float ux, float uy, float uz, int c) {
-  if constexpr (FMT == kRecF32) {
-    return grid_sample_nb(g, ux, uy, uz, c);
-  } else {
-    const bool inb = (ux >= 0.f) & (ux <= g.mx) & (uy >= 0.f) & (uy <= g.my) & (uz >= 0.f) & (uz <= g.mz);
-    const float vx = fminf(fmaxf(ux, 0.f), g.mx), vy = fminf(fmaxf(uy, 0.f), g.my), vz = fminf(fmaxf(uz, 0.f), g.mz);
-    const float fx = floorf(vx), fy = floorf(vy), fz = floorf(vz);   // the padding layer holds the upper faces
-    const size_t ri = rec_index(g.cx, g.cy, g.cz, c, (int)fx, (int)fy, (int)fz);
-    if (!lg_check(g.check, c >= 0 && c < g.nc && ri < g.n_rec, kChkGridRecord)) return g.penalty;
-    const float e = lerp16<FMT>(__ldg(reinterpret_cast<const uint4*>(g.coef) + ri), vx - fx, vy - fy, vz - fz);
-    return inb ? e : g.penalty;
-  }
+__device__ __forceinline__ DockPoint dock_point(const GridView& g, float ux, float uy, float uz) {
+  constexpr bool kClamp = FMT == kRecF32;
+  const float tx = __fadd_rz(kClamp ? fminf(ux, g.lx) : ux, kFloorMagic);
+  const float ty = __fadd_rz(kClamp ? fminf(uy, g.ly) : uy, kFloorMagic);
+  const float tz = __fadd_rz(kClamp ? fminf(uz, g.lz) : uz, kFloorMagic);
+  return {ux, uy, uz, __float_as_uint(tx), __float_as_uint(ty), __float_as_uint(tz),
+          ux - (tx - kFloorMagic), uy - (ty - kFloorMagic), uz - (tz - kFloorMagic)};
 }
 
-// 16-bit record samplers with the channel's record base computed by the
-// caller (chan_base16, once per atom): a sample then forms its address from
-// a 32-bit in-channel cell index with one wide multiply-add instead of a
-// 64-bit record index. Same records, same arithmetic, same results as
-// grid_sample_fmt. Measured on GB300 (screen20k docking kernel): FP16
-// 45.65 -> 45.11 ms, BF16 47.13 -> 46.06 ms. The same change to the FP32
-// sampler made it 1.5% slower (more spills in the 8-CTA build), so FP32
-// records keep grid_sample.
-__device__ __forceinline__ const unsigned char* chan_base16(const GridView& g, int c) {
-  return reinterpret_cast<const unsigned char*>(g.coef) + (size_t)c * g.cz * g.cy * g.cx * 16;
+// Two points at once, FP32 records.
+__device__ __forceinline__ void dock_points2(const GridView& g, float2 x, float2 y, float2 z, DockPoint& p,
+                                             DockPoint& q) {
+  const float2 m = make_float2(kFloorMagic, kFloorMagic);
+  const float2 tx = add2_rz(make_float2(fminf(x.x, g.lx), fminf(x.y, g.lx)), m);
+  const float2 ty = add2_rz(make_float2(fminf(y.x, g.ly), fminf(y.y, g.ly)), m);
+  const float2 tz = add2_rz(make_float2(fminf(z.x, g.lz), fminf(z.y, g.lz)), m);
+  const float2 dx = sub2(x, sub2(tx, m)), dy = sub2(y, sub2(ty, m)), dz = sub2(z, sub2(tz, m));
+  p = {x.x, y.x, z.x, __float_as_uint(tx.x), __float_as_uint(ty.x), __float_as_uint(tz.x), dx.x, dy.x, dz.x};
+  q = {x.y, y.y, z.y, __float_as_uint(tx.y), __float_as_uint(ty.y), __float_as_uint(tz.y), dx.y, dy.y, dz.y};
 }
 
+__device__ __forceinline__ bool dock_in(const GridView& g, const DockPoint& p) {
+  return (__float_as_uint(p.ux) <= g.hx) & (__float_as_uint(p.uy) <= g.hy) & (__float_as_uint(p.uz) <= g.hz);
+}
+
+// Channel c's records: for coefficient records (at most 2^31 of them) an
+// index offset, for 16-bit ones (padded, possibly more) an address.
 template <int FMT>
-__device__ __forceinline__ float grid_sample16_cb(const GridView& g, const unsigned char* cb, float ux, float uy,
-                                                  float uz, int c) {
-  static_assert(FMT != kRecF32, "16-bit records only");
-  const bool inb = (ux >= 0.f) & (ux <= g.mx) & (uy >= 0.f) & (uy <= g.my) & (uz >= 0.f) & (uz <= g.mz);
-  float e = g.penalty;
-  if (inb) {
-    const float fx = floorf(ux), fy = floorf(uy), fz = floorf(uz);   // the padding layer holds the upper faces
-    const int ix = (int)fx, iy = (int)fy, iz = (int)fz;
-    const float dx = ux - fx, dy = uy - fy, dz = uz - fz;
-    const unsigned li = (unsigned)((iz * g.cy + iy) * g.cx + ix);
-    if constexpr (LIGEN_CHECKED) {
-      const size_t ri = rec_index(g.cx, g.cy, g.cz, c, ix, iy, iz);
-      if (!lg_check(g.check, c >= 0 && c < g.nc && ri < g.n_rec, kChkGridRecord)) return g.penalty;
+struct DockChannel {
+  unsigned off;
+  const unsigned char* base;
+  __device__ __forceinline__ DockChannel(const GridView& g, int c) {
+    if constexpr (FMT == kRecF32) {
+      off = (unsigned)c * g.cells - g.bias;
+      base = nullptr;
+    } else {
+      off = 0u;   // the bias is subtracted as a constant operand
+      base = reinterpret_cast<const unsigned char*>(g.coef) + (size_t)c * g.cz * g.cy * g.cx * 16;
     }
-    const uint4 v = __ldg(reinterpret_cast<const uint4*>(cb) + li);
-    e = lerp16<FMT>(v, dx, dy, dz);
   }
-  return e;
+};
+
+// Energy at a point; with GUARD any point (the first record is loaded for one
+// outside the box, without a branch), else one for which dock_in holds.
+template <int FMT, bool GUARD = false>
+__device__ __forceinline__ float dock_energy(const GridView& g, const DockChannel<FMT>& ch, const DockPoint& p, int c) {
+  const bool in = !GUARD || dock_in(g, p);
+  const unsigned cell = (p.bz * g.cy + p.by) * g.cx + p.bx;
+  if constexpr (FMT == kRecF32) {
+    const unsigned ri = in ? cell + ch.off : 0u;
+    if (!lg_check(g.check, c >= 0 && c < g.nc && ri < g.n_rec, kChkGridRecord)) return g.penalty;
+    float a[8];
+    ld_global_v8_na(g.coef + (size_t)ri * 8, a);
+    const float t1 = fmaf(p.dz, a[7], a[4]);
+    float t2 = fmaf(p.dy, t1, a[1]);
+    t2 = fmaf(p.dz, a[5], t2);
+    const float t3 = fmaf(p.dz, a[6], a[2]);
+    float e = fmaf(p.dz, a[3], a[0]);
+    e = fmaf(p.dy, t3, e);
+    e = fmaf(p.dx, t2, e);
+    return in ? e : g.penalty;
+  } else {
+    const unsigned ri = in ? cell - g.bias : 0u;
+    if (!lg_check(g.check, c >= 0 && c < g.nc && (size_t)c * g.cz * g.cy * g.cx + ri < g.n_rec, kChkGridRecord))
+      return g.penalty;
+    const float e = lerp16<FMT>(__ldg(reinterpret_cast<const uint4*>(ch.base) + ri), p.dx, p.dy, p.dz);
+    return in ? e : g.penalty;
+  }
 }
 
 // Value and gradient (per grid unit) of channel `c` at grid-unit position u:

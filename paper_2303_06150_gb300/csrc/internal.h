@@ -174,7 +174,9 @@ size_t dock_smem_bytes(int max_atoms, int max_rot, int max_frag, int rpc);
 int dock_pick_lanes(const int32_t* h_atom_off, const int32_t* h_rot_off, int L, int R, int n_rigid, int n_theta,
                     int passes, int fmt, int sms);
 bool dock_lanes_supported(int lanes);
-bool dock_shape_supported(int lanes, int fmt);
+// A grid axis of 2^23 cells or more: docked by the 8-lane shapes only.
+inline bool dock_big(const GridView& g) { return g.mx >= kFloorMagic || g.my >= kFloorMagic || g.mz >= kFloorMagic; }
+bool dock_shape_supported(int lanes, int fmt, bool big);
 // grid_ctas: CTAs of a persistent launch (ignored when a.queue is NULL).
 // set_attr: set the kernel's dynamic shared-memory limit first (false when
 // dock_occupancy already did, e.g. before a stream capture).
@@ -182,9 +184,9 @@ cudaError_t launch_dock(const DockArgs& a, int grid_ctas, cudaStream_t s, bool s
 // The kernel of (lanes, n_theta) accepts up to `smem` bytes of dynamic
 // shared memory from now on (a per-kernel setting: set the largest value any
 // pending launch of that kernel needs).
-cudaError_t dock_set_smem_limit(int lanes, int n_theta, int fmt, size_t smem);
+cudaError_t dock_set_smem_limit(int lanes, int n_theta, int fmt, bool big, size_t smem);
 // Resident CTAs per SM for a launch with `smem` bytes (within the limit).
-cudaError_t dock_occupancy(int lanes, int n_theta, int fmt, int rpc, size_t smem, int* blocks_per_sm);
+cudaError_t dock_occupancy(int lanes, int n_theta, int fmt, bool big, int rpc, size_t smem, int* blocks_per_sm);
 cudaError_t launch_topk(const TopkArgs& a, cudaStream_t s);
 cudaError_t launch_score(const ScoreArgs& a, cudaStream_t s);
 // Pose-per-lane scoring of the ligands a.list[0 .. n_list) (all of them at

@@ -36,7 +36,7 @@ namespace {
 constexpr unsigned kFull = 0xffffffffu;
 
 struct SmemLayout {
-  float4* sx;       // [max_atoms]
+  float4* sx;       // [max_atoms] two float4 per pair of atoms: (x0, x1, y0, y1), (z0, z1, type0, type1)
   float* cx;        // [max_atoms][rpc]
   float* cy;
   float* cz;
@@ -52,7 +52,7 @@ __host__ __device__ inline size_t align16(size_t v) { return (v + 15) & ~(size_t
 __host__ __device__ inline size_t carve(int max_atoms, int max_rot, int max_frag, int rpc,
                                         unsigned char* base, SmemLayout* L) {
   size_t off[9];
-  const size_t bytes[9] = {(size_t)max_atoms * 16, (size_t)max_atoms * rpc * 4, (size_t)max_atoms * rpc * 4,
+  const size_t bytes[9] = {(size_t)(max_atoms + 1) / 2 * 32, (size_t)max_atoms * rpc * 4, (size_t)max_atoms * rpc * 4,
                            (size_t)max_atoms * rpc * 4, (size_t)max_rot * 4, (size_t)max_rot * 2,
                            (size_t)max_rot * rpc, (size_t)max_frag, (size_t)max_rot * 4};
   size_t o = 0;
@@ -65,6 +65,10 @@ __host__ __device__ inline size_t carve(int max_atoms, int max_rot, int max_frag
     L->stouch = (uint32_t*)(base + off[8]);
   }
   return o;
+}
+
+__device__ __forceinline__ int atom_type(const SmemLayout& S, int i) {
+  return reinterpret_cast<const int*>(S.sx)[(i >> 1) * 8 + 6 + (i & 1)];
 }
 
 // Increment a lane evaluates in the sweep slot that starts at `base`: its
@@ -93,7 +97,8 @@ __device__ __forceinline__ void group_argmax(float& s, int& idx) {
 // One work item: ligand l, restarts [chunk * rpc, chunk * rpc + rpc).
 // COUNT: also add the samples the item's restarts needed to a.samples (a
 // separate instantiation, so the plain kernel carries no counting).
-template <int G, int SLOTS, int FMT, bool COUNT, int UT>
+// BIG: a grid axis of 2^23 cells or more, beyond the packed sampler's floor.
+template <int G, int SLOTS, int FMT, bool COUNT, int UT, bool BIG>
 __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S, int l, int chunk) {
   const int rpc = a.rpc;
   const int tid = threadIdx.x;
@@ -103,7 +108,11 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
   const int n = a.lig.rot_off[l + 1] - r0;
   if (!lg_check(a.grid.check, N <= a.max_atoms && n <= a.max_rot, kChkItemShape)) return;   // uniform
 
-  for (int i = tid; i < N; i += blockDim.x) S.sx[i] = a.pk.xc[a0 + i];
+  for (int i = tid; i < N + (N & 1); i += blockDim.x) {   // an odd ligand's last pair repeats its last atom
+    const float4 X = a.pk.xc[a0 + min(i, N - 1)];
+    float* d = reinterpret_cast<float*>(S.sx) + (i >> 1) * 8 + (i & 1);
+    d[0] = X.x; d[2] = X.y; d[4] = X.z; d[6] = X.w;
+  }
   for (int b = tid; b < n; b += blockDim.x) {
     S.sb[b] = a.pk.binfo[r0 + b];
     S.stouch[b] = a.pk.touch[r0 + b];
@@ -156,7 +165,7 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
     o[k] = (t - a.origin[k]) * a.inv_h;
   }
 
-  constexpr int kRigidUnroll = UT > 1 ? 8 : 4;
+  constexpr int kRigidUnroll = UT > 1 ? 8 : 4, kRigidPairs = UT > 1 ? 4 : 1;
   // ---- rigid stage: lane `sub` scores cube rotations sub, sub+G, ...
   float best = -INFINITY;
   int kb = 0;
@@ -165,16 +174,45 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
     cube_mat(k, Gk);
     mat3mul(M, Gk, Mk);
     float acc = 0.f;
+    if constexpr (FMT == kRecF32 && !BIG) {   // two atoms per packed instruction
+      const float2 m0 = make_float2(Mk[0], Mk[0]), m1 = make_float2(Mk[1], Mk[1]), m2 = make_float2(Mk[2], Mk[2]);
+      const float2 m3 = make_float2(Mk[3], Mk[3]), m4 = make_float2(Mk[4], Mk[4]), m5 = make_float2(Mk[5], Mk[5]);
+      const float2 m6 = make_float2(Mk[6], Mk[6]), m7 = make_float2(Mk[7], Mk[7]), m8 = make_float2(Mk[8], Mk[8]);
+      const float2 o0 = make_float2(o[0], o[0]), o1 = make_float2(o[1], o[1]), o2 = make_float2(o[2], o[2]);
+#pragma unroll kRigidPairs
+      for (int i = 0; i < N; i += 2) {
+        const float4 A = S.sx[i], B = S.sx[i + 1];
+        const float2 X = make_float2(A.x, A.y), Y = make_float2(A.z, A.w), Z = make_float2(B.x, B.y);
+        const int c0 = __float_as_int(B.z), c1 = __float_as_int(B.w);
+        DockPoint p, q;
+        dock_points2(grid, fma2(m0, X, fma2(m1, Y, fma2(m2, Z, o0))), fma2(m3, X, fma2(m4, Y, fma2(m5, Z, o1))),
+                     fma2(m6, X, fma2(m7, Y, fma2(m8, Z, o2))), p, q);
+        float e0 = grid.penalty, e1 = grid.penalty;
+        if constexpr (UT > 1) {
+          e0 = dock_energy<FMT, true>(grid, DockChannel<FMT>(grid, c0), p, c0);
+          e1 = dock_energy<FMT, true>(grid, DockChannel<FMT>(grid, c1), q, c1);
+        } else {
+          if (dock_in(grid, p)) e0 = dock_energy<FMT>(grid, DockChannel<FMT>(grid, c0), p, c0);
+          if (dock_in(grid, q)) e1 = dock_energy<FMT>(grid, DockChannel<FMT>(grid, c1), q, c1);
+        }
+        acc -= e0;
+        if (i + 1 < N) acc -= e1;
+      }
+    } else {
 #pragma unroll kRigidUnroll
-    for (int i = 0; i < N; ++i) {
-      const float4 X = S.sx[i];
-      const float ux = fmaf(Mk[0], X.x, fmaf(Mk[1], X.y, fmaf(Mk[2], X.z, o[0])));
-      const float uy = fmaf(Mk[3], X.x, fmaf(Mk[4], X.y, fmaf(Mk[5], X.z, o[1])));
-      const float uz = fmaf(Mk[6], X.x, fmaf(Mk[7], X.y, fmaf(Mk[8], X.z, o[2])));
-      const int c = __float_as_int(X.w);
-      if constexpr (UT > 1) acc -= grid_sample_nb_fmt<FMT>(grid, ux, uy, uz, c);
-      else if constexpr (FMT == kRecF32) acc -= grid_sample(grid, ux, uy, uz, c);
-      else acc -= grid_sample16_cb<FMT>(grid, chan_base16(grid, c), ux, uy, uz, c);
+      for (int i = 0; i < N; ++i) {
+        const float* d = reinterpret_cast<const float*>(S.sx) + (i >> 1) * 8 + (i & 1);
+        const float3 X = make_float3(d[0], d[2], d[4]);
+        const int c = __float_as_int(d[6]);
+        const DockPoint p = dock_point<FMT>(grid, fmaf(Mk[0], X.x, fmaf(Mk[1], X.y, fmaf(Mk[2], X.z, o[0]))),
+                                            fmaf(Mk[3], X.x, fmaf(Mk[4], X.y, fmaf(Mk[5], X.z, o[1]))),
+                                            fmaf(Mk[6], X.x, fmaf(Mk[7], X.y, fmaf(Mk[8], X.z, o[2]))));
+        float e = grid.penalty;
+        if constexpr (BIG) e = grid_sample_fmt<FMT>(grid, p.ux, p.uy, p.uz, c);
+        else if constexpr (UT > 1) e = dock_energy<FMT, true>(grid, DockChannel<FMT>(grid, c), p, c);
+        else if (dock_in(grid, p)) e = dock_energy<FMT>(grid, DockChannel<FMT>(grid, c), p, c);
+        acc -= e;
+      }
     }
     if (acc > best) { best = acc; kb = k; }
   }
@@ -189,7 +227,8 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
     cube_mat(kb, Gk);
     mat3mul(M, Gk, Mk);
     for (int i = sub; i < N; i += G) {
-      const float4 X = S.sx[i];
+      const float* d = reinterpret_cast<const float*>(S.sx) + (i >> 1) * 8 + (i & 1);
+      const float3 X = make_float3(d[0], d[2], d[4]);
       S.cx[i * rpc + rr] = fmaf(Mk[0], X.x, fmaf(Mk[1], X.y, fmaf(Mk[2], X.z, o[0])));
       S.cy[i * rpc + rr] = fmaf(Mk[3], X.x, fmaf(Mk[4], X.y, fmaf(Mk[5], X.z, o[1])));
       S.cz[i * rpc + rr] = fmaf(Mk[6], X.x, fmaf(Mk[7], X.y, fmaf(Mk[8], X.z, o[2])));
@@ -263,7 +302,8 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
 #pragma unroll
             for (int q = 0; q < UT; ++q) {
               const int i = S.sfrag[off + min(t0 + q, m_live - 1)];   // past the end: the last atom again, not added
-              const int c = __float_as_int(S.sx[i].w);
+              const int c = atom_type(S, i);
+              const DockChannel<FMT> ch(grid, c);
               const float dx = S.cx[i * rpc + rr] - vx;
               const float dy = S.cy[i * rpc + rr] - vy;
               const float dz = S.cz[i * rpc + rr] - vz;
@@ -273,10 +313,10 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
               const float qx = ky * dz - kz * dy, qy = kz * dx - kx * dz, qz = kx * dy - ky * dx;
 #pragma unroll
               for (int s = 0; s < SLOTS; ++s) {
-                const float ux = fmaf(ex, cs[s], fmaf(qx, sn[s], px));
-                const float uy = fmaf(ey, cs[s], fmaf(qy, sn[s], py));
-                const float uz = fmaf(ez, cs[s], fmaf(qz, sn[s], pz));
-                e[q][s] = grid_sample_nb_fmt<FMT>(grid, ux, uy, uz, c);
+                const DockPoint p = dock_point<FMT>(grid, fmaf(ex, cs[s], fmaf(qx, sn[s], px)),
+                                                    fmaf(ey, cs[s], fmaf(qy, sn[s], py)),
+                                                    fmaf(ez, cs[s], fmaf(qz, sn[s], pz)));
+                e[q][s] = dock_energy<FMT, true>(grid, ch, p, c);
               }
             }
 #pragma unroll
@@ -289,8 +329,8 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
         } else {
           for (int t = 0; t < m_live; ++t) {
             const int i = S.sfrag[off + t];
-            const int c = __float_as_int(S.sx[i].w);
-            const unsigned char* cb = FMT == kRecF32 ? nullptr : chan_base16(grid, c);   // 16-bit records
+            const int c = atom_type(S, i);
+            const DockChannel<FMT> ch(grid, c);
             const float dx = S.cx[i * rpc + rr] - vx;
             const float dy = S.cy[i * rpc + rr] - vy;
             const float dz = S.cz[i * rpc + rr] - vz;
@@ -298,9 +338,32 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
             const float px = fmaf(kx, kd, vx), py = fmaf(ky, kd, vy), pz = fmaf(kz, kd, vz);
             const float ex = fmaf(-kx, kd, dx), ey = fmaf(-ky, kd, dy), ez = fmaf(-kz, kd, dz);
             const float qx = ky * dz - kz * dy, qy = kz * dx - kx * dz, qz = kx * dy - ky * dx;
-            if constexpr (FMT != kRecF32) {
-              // two increments per packed instruction (measured: 0.5% faster
-              // with 16-bit records, 1% slower with FP32 records)
+            if constexpr (FMT == kRecF32 && !BIG) {   // two increments per packed instruction
+              float e[SLOTS];
+#pragma unroll
+              for (int s = 0; s < SLOTS; ++s) e[s] = grid.penalty;
+#pragma unroll
+              for (int s = 0; s + 1 < SLOTS; s += 2) {
+                const float2 cc = make_float2(cs[s], cs[s + 1]), ss = make_float2(sn[s], sn[s + 1]);
+                DockPoint p, q;
+                dock_points2(grid, fma2(make_float2(ex, ex), cc, fma2(make_float2(qx, qx), ss, make_float2(px, px))),
+                             fma2(make_float2(ey, ey), cc, fma2(make_float2(qy, qy), ss, make_float2(py, py))),
+                             fma2(make_float2(ez, ez), cc, fma2(make_float2(qz, qz), ss, make_float2(pz, pz))), p, q);
+                if (dock_in(grid, q)) e[s + 1] = dock_energy<FMT>(grid, ch, q, c);
+                if (dock_in(grid, p)) e[s] = dock_energy<FMT>(grid, ch, p, c);
+              }
+              if constexpr (SLOTS % 2 == 1) {
+                const DockPoint p =
+                    dock_point<FMT>(grid, fmaf(ex, cs[SLOTS - 1], fmaf(qx, sn[SLOTS - 1], px)),
+                                    fmaf(ey, cs[SLOTS - 1], fmaf(qy, sn[SLOTS - 1], py)),
+                                    fmaf(ez, cs[SLOTS - 1], fmaf(qz, sn[SLOTS - 1], pz)));
+                if (dock_in(grid, p)) e[SLOTS - 1] = dock_energy<FMT>(grid, ch, p, c);
+              }
+#pragma unroll
+              for (int s = 0; s < SLOTS; ++s) acc[s] -= e[s];
+            } else {
+              // the rotation in pairs only: cells and fractions in pairs too
+              // keep more registers live and were 1-3% slower
               float ux[SLOTS], uy[SLOTS], uz[SLOTS];
 #pragma unroll
               for (int s = 0; s + 1 < SLOTS; s += 2) {
@@ -316,14 +379,12 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
                 uz[SLOTS - 1] = fmaf(ez, cs[SLOTS - 1], fmaf(qz, sn[SLOTS - 1], pz));
               }
 #pragma unroll
-              for (int s = 0; s < SLOTS; ++s) acc[s] -= grid_sample16_cb<FMT>(grid, cb, ux[s], uy[s], uz[s], c);
-            } else {
-#pragma unroll
               for (int s = 0; s < SLOTS; ++s) {
-                const float ux = fmaf(ex, cs[s], fmaf(qx, sn[s], px));
-                const float uy = fmaf(ey, cs[s], fmaf(qy, sn[s], py));
-                const float uz = fmaf(ez, cs[s], fmaf(qz, sn[s], pz));
-                acc[s] -= grid_sample_fmt<FMT>(grid, ux, uy, uz, c);
+                const DockPoint p = dock_point<FMT>(grid, ux[s], uy[s], uz[s]);
+                float e = grid.penalty;
+                if constexpr (BIG) e = grid_sample_fmt<FMT>(grid, p.ux, p.uy, p.uz, c);
+                else if (dock_in(grid, p)) e = dock_energy<FMT>(grid, ch, p, c);
+                acc[s] -= e;
               }
             }
           }
@@ -358,7 +419,8 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
       }
       __syncwarp();
       if (sub == 0) {
-        S.scnt[b * rpc + rr] = (uint8_t)((S.scnt[b * rpc + rr] + jb) % nt);
+        const int cnt = S.scnt[b * rpc + rr] + jb;   // both below nt
+        S.scnt[b * rpc + rr] = (uint8_t)(cnt >= nt ? cnt - nt : cnt);
         if (trace) trace[1 + p * n + b] = (int16_t)jb;
       }
       // a turn dirties the bonds it touches; the bond itself is clean either way
@@ -373,12 +435,13 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
   if constexpr (UT > 1) {
 #pragma unroll 4
     for (int i = sub % FG; i < N; i += FG)
-      acc -= grid_sample_nb_fmt<FMT>(grid, S.cx[i * rpc + rr], S.cy[i * rpc + rr], S.cz[i * rpc + rr],
-                                     __float_as_int(S.sx[i].w));
+      acc -= dock_energy<FMT, true>(
+          grid, DockChannel<FMT>(grid, atom_type(S, i)),
+          dock_point<FMT>(grid, S.cx[i * rpc + rr], S.cy[i * rpc + rr], S.cz[i * rpc + rr]), atom_type(S, i));
   } else {
     for (int i = sub; i < N; i += G)
       acc -= grid_sample_fmt<FMT>(grid, S.cx[i * rpc + rr], S.cy[i * rpc + rr], S.cz[i * rpc + rr],
-                                  __float_as_int(S.sx[i].w));
+                                  atom_type(S, i));
   }
 #pragma unroll
   for (int off = 1; off < FG; off <<= 1) acc += __shfl_xor_sync(kFull, acc, off);
@@ -386,7 +449,7 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
     long long v = (active && sub == 0) ? needed : 0;
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(kFull, v, o);
-    if ((tid & 31) == 0) atomicAdd(&a.samples[blockIdx.x % kSampleSlots], (unsigned long long)v);
+    if ((tid & 31) == 0 && a.samples) atomicAdd(&a.samples[blockIdx.x % kSampleSlots], (unsigned long long)v);
   }
   if (a.coords && active) {   // debug output: the positions the final score sampled
     float* cd = a.coords + 3 * ((size_t)a.R * a0 + (size_t)r * N);
@@ -406,15 +469,15 @@ __device__ __forceinline__ void dock_item(const DockArgs& a, const SmemLayout& S
 }
 
 // MINB: resident CTAs asked of the register allocator (1: no request).
-// 8-lane shapes come in four builds: 8 CTAs (64 registers, some spill to
-// local memory), 7 (72 registers), 6 (~80) and unconstrained (~100, 4 CTAs).
-// More CTAs pay only while their shared memory leaves L1 room for the
-// spills and the gathers: measured on GB300, the screening library (~20 KB
-// per CTA) docks fastest with 8 CTAs, the bimodal one (27.6 KB per CTA) with
-// 7 (8 leave under 48 KB of L1 and run 60% slower; 6 CTAs 9%, the
-// unconstrained build 42%).
+// 8-lane shapes come in four builds: 8 CTAs (64 registers; 16-bit records
+// and two-slot shapes only, see build_ctas), 7 (72 registers), 6 (~80) and
+// unconstrained (4-5 CTAs). The gathers' latency wants many warps (12,000
+// screening ligands, FP32: 7 CTAs 23.0 ms, 6 CTAs 27.5), but more CTAs pay
+// only while their shared memory leaves L1 room for the spills and the
+// 16-bit gathers: the bimodal library (27.6 KB per CTA) docks fastest with 7
+// (FP16: 8 leave under 48 KB of L1, 17.0 against 11.2 ms).
 // launch_dock takes the largest count whose CTAs fit kCtaSmemBudget.
-template <int G, int SLOTS, int FMT, bool COUNT, int MINB, int UT>
+template <int G, int SLOTS, int FMT, bool COUNT, int MINB, int UT, bool BIG = false>
 __global__ void __launch_bounds__(128, MINB) dock_kernel(const DockArgs a) {
   extern __shared__ __align__(16) unsigned char smem[];
   __shared__ int next_item;
@@ -432,7 +495,7 @@ __global__ void __launch_bounds__(128, MINB) dock_kernel(const DockArgs a) {
     const int li = item / a.chunks;
     const int l = a.list ? a.list[li] : li;
     if (a.pk.status[l] == 0)   // uniform over the CTA
-      dock_item<G, SLOTS, FMT, COUNT, UT>(a, S, l, item - li * a.chunks);
+      dock_item<G, SLOTS, FMT, COUNT, UT, BIG>(a, S, l, item - li * a.chunks);
     if (!a.queue) break;
     __syncthreads();   // shared memory is reused by the next item
   }
@@ -450,13 +513,18 @@ using KernelFn = void (*)(DockArgs);
 
 
 // Resident CTAs asked of the register allocator: `ctas` for the 8-lane
-// shapes (see dock_kernel); 4 for the 16-lane ones (128 registers) and 3 for
+// shapes (see dock_kernel; at most 7 with five FP32 gathers in flight, whose
+// 64-register build spills enough to lose: 12,000 screening ligands 24.5
+// against 23.0 ms); 4 for the 16-lane ones (128 registers) and 3 for
 // the 32-lane ones (168). Left to itself the allocator takes 200-254 for the
 // gathers in flight, two CTAs per SM: that is 15-20% faster while one CTA
 // per SM runs (5 screening ligands 92 against 111 us with four) and 20-30%
 // slower from a few dozen ligands on (160 ligands on 16 lanes 731 against
 // 553 us).
-constexpr int build_ctas(int G, int ctas) { return G == 8 ? ctas : G == 16 ? 4 : G == 32 ? 3 : 1; }
+constexpr int build_ctas(int G, int SLOTS, int fmt, int ctas) {
+  if (G == 8) return ctas == 8 && SLOTS > 2 && fmt == kRecF32 ? 7 : ctas;
+  return G == 16 ? 4 : G == 32 ? 3 : 1;
+}
 
 // Instantiated (G, SLOTS, record format) shapes; G * SLOTS increments per
 // chunk of the sweep.
@@ -465,8 +533,8 @@ struct Shape {
   KernelFn fn[2][4];   // [counts the samples needed][build: 8, 7, 6 CTAs, unconstrained]
 };
 #define LG_BUILDS(G, S, F, C, U)                                                                      \
-  {dock_kernel<G, S, F, C, build_ctas(G, 8), U>, dock_kernel<G, S, F, C, build_ctas(G, 7), U>,         \
-   dock_kernel<G, S, F, C, build_ctas(G, 6), U>, dock_kernel<G, S, F, C, build_ctas(G, 1), U>}
+  {dock_kernel<G, S, F, C, build_ctas(G, S, F, 8), U>, dock_kernel<G, S, F, C, build_ctas(G, S, F, 7), U>,         \
+   dock_kernel<G, S, F, C, build_ctas(G, S, F, 6), U>, dock_kernel<G, S, F, C, build_ctas(G, S, F, 1), U>}
 // The counting kernel only serves untimed calls: one build for all four.
 #define LG_COUNTING(G, S, F, U)                                                                          \
   {dock_kernel<G, S, F, true, 1, U>, dock_kernel<G, S, F, true, 1, U>, dock_kernel<G, S, F, true, 1, U>,  \
@@ -507,6 +575,15 @@ const Shape kShapes[] = {
 #undef LG_SHAPE
 #undef LG_COUNTING
 #undef LG_BUILDS
+// Grids with an axis of 2^23 cells or more: one 8-lane shape per format,
+// counting or not.
+#define LG_BIG(F)                                                                                        \
+  {8, 5, F, {{dock_kernel<8, 5, F, true, 1, 1, true>, dock_kernel<8, 5, F, true, 1, 1, true>,            \
+              dock_kernel<8, 5, F, true, 1, 1, true>, dock_kernel<8, 5, F, true, 1, 1, true>},           \
+             {dock_kernel<8, 5, F, true, 1, 1, true>, dock_kernel<8, 5, F, true, 1, 1, true>,            \
+              dock_kernel<8, 5, F, true, 1, 1, true>, dock_kernel<8, 5, F, true, 1, 1, true>}}}
+const Shape kBigShapes[] = {LG_BIG(kRecF32), LG_BIG(kRecF16), LG_BIG(kRecBF16)};
+#undef LG_BIG
 
 // Shared memory the resident CTAs may take together (of the SM's 256 KB of
 // L1 and shared memory), and the build for a CTA of `smem` bytes: the one
@@ -523,7 +600,8 @@ int build_for(size_t smem) {
 // The instantiation for G lanes, n_theta increments and record format: the
 // fewest slots that cover n_theta in one chunk, else the largest (several
 // chunks).
-const Shape* pick_shape(int G, int n_theta, int fmt) {
+const Shape* pick_shape(int G, int n_theta, int fmt, bool big) {
+  if (big) return G == 8 ? &kBigShapes[fmt] : nullptr;
   const Shape* best = nullptr;
   for (const Shape& sh : kShapes) {
     if (sh.G != G || sh.FMT != fmt) continue;
@@ -539,7 +617,7 @@ const Shape* pick_shape(int G, int n_theta, int fmt) {
 // Sweep slots a group computes per moving atom: n_theta rounded up to whole
 // lanes and chunks.
 int sweep_slots(int G, int n_theta, int fmt) {
-  const Shape* sh = pick_shape(G, n_theta, fmt);
+  const Shape* sh = pick_shape(G, n_theta, fmt, false);
   const int per = sh->G * sh->SLOTS;
   return (n_theta + per - 1) / per * per;
 }
@@ -554,23 +632,23 @@ int sweep_slots(int G, int n_theta, int fmt) {
 // rate) and the shortest taken. Work counts the candidate samples of the
 // rigid stage and of full sweeps of n_theta = 36 slots, (N + 4) / 4 moving
 // atoms a bond (plan_groups' estimate) and a constant per restart for the
-// rest. Constants fitted to launches of 1-20,000 screening, 1-5,000 bimodal
-// and 32-3,000 small ligands on GB300, longest ligand first; measured
-// docking kernel (us), chosen one first:
+// rest. Constants fitted to launches of 1-20,000 screening, 5-1,000 bimodal
+// and 32-20,000 small ligands on GB300, longest ligand first; measured
+// docking kernel (us), * the one chosen:
 //                        5 ligands   20        80        160       320
-//   screening   8 lanes  430         311       354       621       817*
-//              16 lanes  145         125       279*      553*      1454
-//              32 lanes  92*         115*      397       797       2123
-//   bimodal     8 lanes  788         866       1032      1202      1325*
-//              16 lanes  256         309       434*      850*      1632
-//              32 lanes  164*        242*      590       1196      2312
+//   screening   8 lanes  303         217       272       483*      702*
+//              16 lanes  129         111*      240*      467       920
+//              32 lanes  107*        117       414       831       1649
+//   bimodal     8 lanes  547         618       752       922       1087*
+//              16 lanes  221         266*      377*      725*      1391
+//              32 lanes  184*        229       625       1280      2484
 int dock_pick_lanes(const int32_t* h_atom_off, const int32_t* h_rot_off, int L, int R, int n_rigid, int n_theta,
                     int passes, int fmt, int sms) {
   struct Model {
     int lanes;
     double us, us_per_cost, cost_per_us;   // chain: us + us_per_cost * cost; throughput
   };
-  constexpr Model kModels[] = {{8, 50., 0.0135, 1.143e6}, {16, 40., 0.0036, 0.766e6}, {32, 40., 0.0024, 0.522e6}};
+  constexpr Model kModels[] = {{8, 60., 0.0085, 1.294e6}, {16, 42., 0.0030, 0.908e6}, {32, 42., 0.0023, 0.498e6}};
   constexpr double kRestart = 2000.;   // cost of a restart outside its samples
   constexpr int kSms = 152;            // of the measurements
   if ((double)L * R > 400. * sms) return 8;   // fills the chip with any ligands
@@ -596,11 +674,11 @@ int dock_pick_lanes(const int32_t* h_atom_off, const int32_t* h_rot_off, int L, 
 
 bool dock_lanes_supported(int G) { return G == 2 || G == 4 || G == 8 || G == 16 || G == 32; }
 
-bool dock_shape_supported(int G, int fmt) { return pick_shape(G, 36, fmt) != nullptr; }
+bool dock_shape_supported(int G, int fmt, bool big) { return pick_shape(G, 36, fmt, big) != nullptr; }
 
 cudaError_t launch_dock(const DockArgs& a, int grid_ctas, cudaStream_t s, bool set_attr) {
   if (a.n_items == 0) return cudaSuccess;
-  const Shape* sh = pick_shape(a.lanes, a.n_theta, a.fmt);
+  const Shape* sh = pick_shape(a.lanes, a.n_theta, a.fmt, dock_big(a.grid));
   if (!sh) return cudaErrorInvalidValue;
   const size_t smem = dock_smem_bytes(a.max_atoms, a.max_rot, a.max_frag, a.rpc);
   const KernelFn fn = sh->fn[a.samples != nullptr][build_for(smem)];
@@ -613,8 +691,8 @@ cudaError_t launch_dock(const DockArgs& a, int grid_ctas, cudaStream_t s, bool s
   return cudaGetLastError();
 }
 
-cudaError_t dock_set_smem_limit(int lanes, int n_theta, int fmt, size_t smem) {
-  const Shape* sh = pick_shape(lanes, n_theta, fmt);
+cudaError_t dock_set_smem_limit(int lanes, int n_theta, int fmt, bool big, size_t smem) {
+  const Shape* sh = pick_shape(lanes, n_theta, fmt, big);
   if (!sh) return cudaErrorInvalidValue;
   for (int c = 0; c < 2; ++c)
     for (int o = 0; o < 4; ++o) {
@@ -624,8 +702,8 @@ cudaError_t dock_set_smem_limit(int lanes, int n_theta, int fmt, size_t smem) {
   return cudaSuccess;
 }
 
-cudaError_t dock_occupancy(int lanes, int n_theta, int fmt, int rpc, size_t smem, int* blocks_per_sm) {
-  const Shape* sh = pick_shape(lanes, n_theta, fmt);
+cudaError_t dock_occupancy(int lanes, int n_theta, int fmt, bool big, int rpc, size_t smem, int* blocks_per_sm) {
+  const Shape* sh = pick_shape(lanes, n_theta, fmt, big);
   if (!sh) return cudaErrorInvalidValue;
   return cudaOccupancyMaxActiveBlocksPerMultiprocessor(blocks_per_sm, sh->fn[0][build_for(smem)], rpc * lanes,
                                                        smem);

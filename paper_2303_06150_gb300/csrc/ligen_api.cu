@@ -278,6 +278,15 @@ GridView make_view(const ligen_grid_t* g, const float* coef, float penalty, int 
   v.check = nullptr;
   v.nc = g->nc;
   v.mx = (float)(g->nx - 1); v.my = (float)(g->ny - 1); v.mz = (float)(g->nz - 1);
+  v.lx = std::nextafterf(v.mx, 0.f); v.ly = std::nextafterf(v.my, 0.f); v.lz = std::nextafterf(v.mz, 0.f);
+  auto bits = [](float f) {
+    unsigned b;
+    std::memcpy(&b, &f, sizeof b);
+    return b;
+  };
+  v.hx = bits(v.mx); v.hy = bits(v.my); v.hz = bits(v.mz);
+  v.cells = (unsigned)v.cx * (unsigned)v.cy * (unsigned)v.cz;
+  v.bias = bits(8388608.f) * ((unsigned)v.cy * (unsigned)v.cx + (unsigned)v.cx + 1u);
   v.penalty = penalty;
   return v;
 }
@@ -402,7 +411,7 @@ struct Group {
 // order (group, cost descending, ligand index) comes from a stable
 // counting sort in O(L) (the call waits for it before its first launch).
 void plan_groups(const ligen_ligands_t* g, const ligen_params_t* p, int dev, std::vector<int32_t>& order,
-                 std::vector<Group>& groups, bool single = false) {
+                 std::vector<Group>& groups, bool big, bool single) {
   const int L = g->n_ligands;
   const int nt = 360 / p->torsion_step_deg;
   // the group key (atom class, lanes, restarts per CTA) of every bucket,
@@ -412,7 +421,7 @@ void plan_groups(const ligen_ligands_t* g, const ligen_params_t* p, int dev, std
     std::lock_guard<std::mutex> lk(g_tune_mu);
     for (int b = 0; b < LIGEN_N_BUCKETS; ++b) {
       TuneEntry t = single ? TuneEntry() : g_tune[dev][b];
-      if (!dock_shape_supported(t.lanes, p->grid_format)) t = TuneEntry();   // default shape
+      if (!dock_shape_supported(t.lanes, p->grid_format, big)) t = TuneEntry();   // default shape
       bkey[b] = std::make_tuple(single ? 0 : b / 11, t.lanes, t.rpc);
     }
   }
@@ -629,7 +638,7 @@ int run_bucketed(const DockArgs& base, const std::vector<Group>& groups, int32_t
     size_t& l = limit[gr.lanes];
     l = std::max(l, smem);
   }
-  for (const auto& kv : limit) LG_CUDA(dock_set_smem_limit(kv.first, base.n_theta, base.fmt, kv.second));
+  for (const auto& kv : limit) LG_CUDA(dock_set_smem_limit(kv.first, base.n_theta, base.fmt, dock_big(base.grid), kv.second));
   std::vector<DockArgs> args;
   std::vector<int> ctas;
   for (size_t gi = 0; gi < groups.size(); ++gi) {
@@ -646,7 +655,7 @@ int run_bucketed(const DockArgs& base, const std::vector<Group>& groups, int32_t
     a.max_frag = gr.max_frag;
     const size_t smem = dock_smem_bytes(a.max_atoms, a.max_rot, a.max_frag, a.rpc);
     int b = 0;
-    LG_CUDA(dock_occupancy(a.lanes, a.n_theta, a.fmt, a.rpc, smem, &b));
+    LG_CUDA(dock_occupancy(a.lanes, a.n_theta, a.fmt, dock_big(a.grid), a.rpc, smem, &b));
     if (b < 1) return fail(LIGEN_ERR_UNSUPPORTED, "no CTA of shape (%d lanes, %d restarts) fits an SM", a.lanes, a.rpc);
     ctas.push_back(persistent ? (int)std::min<int64_t>((int64_t)b * nsm, a.n_items) : a.n_items);
     args.push_back(a);
@@ -960,6 +969,8 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     if (params->scores_f64 && ohost) o_out64 = ar.take(8 * (size_t)L * K);
   }
   const bool buckets = params->batching != LIGEN_BATCH_PLAIN && !exhaustive;
+  bool any_big = false;
+  for (int g = 0; g < n_sites; ++g) any_big |= dock_big(make_view(&grids[g], nullptr, 0.f, fmt));
   std::vector<int32_t> order;
   std::vector<Group> groups;
   size_t o_order = 0, o_queue = 0;
@@ -979,8 +990,9 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
   bool longest_first = false;
   if (!buckets && !exhaustive) {
     if ((rc = sm_count(&sms)) != LIGEN_OK) return rc;
-    lanes = dock_pick_lanes(ligands->h_atom_off, ligands->h_rot_off, L, R, params->n_rigid,
-                            360 / params->torsion_step_deg, P, fmt, sms);
+    if (!any_big)
+      lanes = dock_pick_lanes(ligands->h_atom_off, ligands->h_rot_off, L, R, params->n_rigid,
+                              360 / params->torsion_step_deg, P, fmt, sms);
     const int rpc = dock_restarts_per_cta(R, lanes);
     longest_first = L > 1 && (int64_t)L * ((R + rpc - 1) / rpc) > sms;
   }
@@ -1095,7 +1107,7 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
       // is staged before cudaMemcpyAsync returns.
       // planned here, on the first site, while the grid records and the
       // packer run on the device
-      if (groups.empty()) plan_groups(ligands, params, plan_dev, order, groups, params->batching == LIGEN_BATCH_QUEUE);
+      if (groups.empty()) plan_groups(ligands, params, plan_dev, order, groups, any_big, params->batching == LIGEN_BATCH_QUEUE);
       int32_t* d_order = ar.at<int32_t>(o_order);
       LG_CUDA(cudaMemcpyAsync(d_order, order.data(), 4 * order.size(), cudaMemcpyHostToDevice, s));
       if ((rc = run_bucketed(da, groups, d_order, ar.at<int>(o_queue),
@@ -1665,8 +1677,8 @@ int64_t ligen_bucket_size(int32_t max_atoms, int32_t* b, int32_t* sm, int32_t* t
   LG_CUDA(cudaDeviceGetAttribute(&warp, cudaDevAttrWarpSize, dev));
   const int rpc = dock_restarts_per_cta(256, kDefaultLanes);
   const size_t smem = dock_smem_bytes(max_atoms, LIGEN_MAX_ROT, LIGEN_MAX_ROT * (max_atoms / 2), rpc);
-  LG_CUDA(dock_set_smem_limit(kDefaultLanes, 36, kRecF32, smem));
-  LG_CUDA(dock_occupancy(kDefaultLanes, 36, kRecF32, rpc, smem, &blocks));
+  LG_CUDA(dock_set_smem_limit(kDefaultLanes, 36, kRecF32, false, smem));
+  LG_CUDA(dock_occupancy(kDefaultLanes, 36, kRecF32, false, rpc, smem, &blocks));
   const int threads = rpc * kDefaultLanes;
   if (b) *b = blocks;
   if (sm) *sm = nsm;
@@ -1820,7 +1832,7 @@ int ligen_autotune(const ligen_ligands_t* ligands, const ligen_grid_t* grid, con
     float best_ms = 0.f;
     int best = -1;
     for (int c = 0; c < (int)(sizeof kCand / sizeof kCand[0]); ++c) {
-      if (!valid_shape(kCand[c][0], kCand[c][1]) || !dock_shape_supported(kCand[c][0], fmt)) continue;
+      if (!valid_shape(kCand[c][0], kCand[c][1]) || !dock_shape_supported(kCand[c][0], fmt, dock_big(base.grid))) continue;
       DockArgs a = base;
       a.lanes = kCand[c][0];
       a.rpc = kCand[c][1];
@@ -2054,8 +2066,9 @@ extern "C" int ligen_dock_batch_static(const ligen_ligands_t* ligands, const lig
   da.step_deg = params->torsion_step_deg;
   da.n_theta = 360 / params->torsion_step_deg;
   da.passes = params->passes;
-  da.lanes = dock_pick_lanes(ligands->h_atom_off, ligands->h_rot_off, L, R, params->n_rigid, da.n_theta,
-                             params->passes, kRecF32, sms);
+  da.lanes = dock_big(da.grid) ? kDefaultLanes
+                               : dock_pick_lanes(ligands->h_atom_off, ligands->h_rot_off, L, R, params->n_rigid,
+                                                 da.n_theta, params->passes, kRecF32, sms);
   da.rpc = dock_restarts_per_cta(R, da.lanes);
   da.chunks = (R + da.rpc - 1) / da.rpc;
   da.list = nullptr;

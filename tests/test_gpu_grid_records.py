@@ -76,3 +76,22 @@ def test_16_bit_records(shape, fmt):
         e, g = _trilinear(w, u[c], c)
         tol = (10 * 8 + top.max()) * 2.0 ** -24 * g
         assert (np.abs(s[c] + e) <= tol).all(), (c, np.abs(s[c] + e).max())
+
+
+@pytest.mark.parametrize("fmt", ["f32", "f16", "bf16"])
+def test_docking_on_an_axis_of_2_to_the_23_cells(fmt):
+    import torch
+
+    import paper_2303_06150_gb300 as lg
+    nz, R = 2 ** 23 + 1, 64
+    v = torch.rand((nz, 2, 2, 1), generator=torch.Generator("cuda").manual_seed(1), device="cuda") - 0.5
+    G = lg.PocketGrid(v, (0.0, 0.0, 0.0), 1.0)
+    r = lg.dock_batch(_one_atom_ligands(lg, 1), G, restarts=R, torsion_step_deg=30, passes=0, top_k=R, seed=1,
+                      n_rigid=1, jitter=0.5, grid_format=fmt)
+    u = r.poses.cpu().numpy().reshape(R, 7)[:, :3].astype(np.float64)   # z: near 2^22, on multiples of 1/2
+    z0 = int(u[:, 2].min()) - 1
+    part = v[z0:z0 + 4].cpu().numpy()
+    u[:, 2] -= z0
+    e, g = _trilinear(parity.record_values(part, fmt), u, 0)
+    # positions are exact here (origin 0, spacing 1): only the record's and the polynomial's roundings
+    assert (np.abs(r.scores.cpu().numpy()[0] + e) <= 10 * 8 * 2.0 ** -24 * g).all()
