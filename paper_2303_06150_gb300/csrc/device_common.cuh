@@ -502,4 +502,59 @@ __device__ __forceinline__ float grid_sample_grad(const GridView& g, float ux, f
   return e;
 }
 
+// A coefficient record fetched ahead of its use: the scoring and gradient
+// kernels issue the loads of several atoms before they use any. Same cell,
+// fractions and box test as grid_sample; a point outside loads the first
+// record. Adding +0 first makes a coordinate of -0 (poses are given, so it
+// can occur) compare as inside.
+struct FetchedRecord {
+  float a[8];
+  float dx, dy, dz;
+  bool in;
+};
+
+__device__ __forceinline__ FetchedRecord grid_fetch(const GridView& g, float ux, float uy, float uz, int c) {
+  FetchedRecord r;
+  ux += 0.f; uy += 0.f; uz += 0.f;
+  const DockPoint p = dock_point<kRecF32>(g, ux, uy, uz);
+  r.dx = p.dx; r.dy = p.dy; r.dz = p.dz;
+  r.in = dock_in(g, p);
+  const unsigned ri = r.in ? (p.bz * g.cy + p.by) * g.cx + p.bx + DockChannel<kRecF32>(g, c).off : 0u;
+  if (!lg_check(g.check, c >= 0 && c < g.nc && ri < g.n_rec, kChkGridRecord)) {
+    r.in = false;
+    return r;
+  }
+  ld_global_v8_na(g.coef + (size_t)ri * 8, r.a);
+  return r;
+}
+
+__device__ __forceinline__ float fetched_value(const GridView& g, const FetchedRecord& r) {
+  const float t1 = fmaf(r.dz, r.a[7], r.a[4]);
+  float t2 = fmaf(r.dy, t1, r.a[1]);
+  t2 = fmaf(r.dz, r.a[5], t2);
+  const float t3 = fmaf(r.dz, r.a[6], r.a[2]);
+  float e = fmaf(r.dz, r.a[3], r.a[0]);
+  e = fmaf(r.dy, t3, e);
+  e = fmaf(r.dx, t2, e);
+  return r.in ? e : g.penalty;
+}
+
+// The value, and the gradient per grid unit (zero outside).
+__device__ __forceinline__ float fetched_grad(const GridView& g, const FetchedRecord& r, float* gx, float* gy,
+                                              float* gz) {
+  const float t1 = fmaf(r.dz, r.a[7], r.a[4]);
+  float t2 = fmaf(r.dy, t1, r.a[1]);
+  t2 = fmaf(r.dz, r.a[5], t2);
+  const float t3 = fmaf(r.dz, r.a[6], r.a[2]);
+  float e = fmaf(r.dz, r.a[3], r.a[0]);
+  e = fmaf(r.dy, t3, e);
+  e = fmaf(r.dx, t2, e);
+  const float hy = fmaf(r.dx, t1, t3);
+  const float hz = fmaf(r.dx, fmaf(r.dy, r.a[7], r.a[5]), fmaf(r.dy, r.a[6], r.a[3]));
+  *gx = r.in ? t2 : 0.f;   // ax + axy fy + axz fz + axyz fy fz
+  *gy = r.in ? hy : 0.f;   // ay + axy fx + ayz fz + axyz fx fz
+  *gz = r.in ? hz : 0.f;   // az + axz fx + ayz fy + axyz fx fy
+  return r.in ? e : g.penalty;
+}
+
 }  // namespace ligen

@@ -50,7 +50,9 @@ __host__ __device__ inline int fk_fstride(int acap) {
 }
 
 // Bytes of the staged ligand (16-byte multiple); carves it at `base` when S.
-__host__ __device__ inline size_t fk_ligand_carve(int acap, int ncap, unsigned char* base, FkLigand* S) {
+// lists: with the moving-atom lists (fk_stage; fk_load has no use for them).
+__host__ __device__ inline size_t fk_ligand_carve(int acap, int ncap, unsigned char* base, FkLigand* S,
+                                                  bool lists) {
   const int fs = fk_fstride(acap);
   const int n16 = (ncap + 15) / 16 * 16;
   const int a16 = (acap + 15) / 16 * 16;
@@ -58,7 +60,7 @@ __host__ __device__ inline size_t fk_ligand_carve(int acap, int ncap, unsigned c
   const size_t osx = o;  o += (size_t)acap * sizeof(float4);
   const size_t oax = o;  o += (size_t)ncap * sizeof(float4);
   const size_t osb = o;  o += (size_t)n16 * sizeof(uchar4);
-  const size_t osf = o;  o += (size_t)ncap * fs;
+  const size_t osf = o;  o += lists ? (size_t)ncap * fs : 0;
   const size_t oown = o; o += (size_t)a16;
   const size_t opar = o; o += (size_t)n16;
   const size_t oord = o; o += (size_t)n16;

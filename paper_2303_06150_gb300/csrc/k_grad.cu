@@ -356,6 +356,12 @@ __global__ void __launch_bounds__(32 * kGradWarps, 6) refine_kernel(const GradAr
 template <int G>
 struct GL {
   static constexpr int PW = 32 / G;   // poses per warp
+  // Records a lane fetches before it uses the first. With one at a time the
+  // kernel waited on its loads (refining the top 16 poses of 4,000 screening
+  // ligands for 50 steps: 2,090 us, 1,710 with four); three and four differ
+  // by 2-6% either way with 2 or 4 lanes per pose, one lane per pose loses
+  // 19% with three.
+  static constexpr int kAhead = G == 1 ? 4 : 3;
 };
 
 // Shared memory of one warp: transforms [ncap + 1][PW][12]; per-lane bond
@@ -373,7 +379,7 @@ __host__ __device__ inline size_t gl_carve(int acap, int ncap, unsigned char* ba
     *acc = (float*)(base + tb);
     *st = (float*)(base + tb + ab);
   }
-  return tb + ab + sb + fk_ligand_carve(acap, ncap, base ? base + tb + ab + sb : nullptr, S);
+  return tb + ab + sb + fk_ligand_carve(acap, ncap, base ? base + tb + ab + sb : nullptr, S, false);
 }
 
 __device__ __forceinline__ float gl_sum(float v, int G) {
@@ -391,9 +397,10 @@ __device__ float gl_eval(const GradArgs& a, const FkLigand& S, int N, int n, con
   const float rqn = rsqrtf(pose[3] * pose[3] + pose[4] * pose[4] + pose[5] * pose[5] + pose[6] * pose[6]);
   const Quat q = {pose[3] * rqn, pose[4] * rqn, pose[5] * rqn, pose[6] * rqn};
   fk_transforms_group<G>(S, n, pose, q, pose + 7, a.origin, a.inv_h, T + 12 * grp, (size_t)PW * 12, sub);
+  float2* const row = reinterpret_cast<float2*>(acc) + lane * 3;   // this lane's sums of bond b: row + 96 b
   for (int b = 0; b < n; ++b)
 #pragma unroll
-    for (int e = 0; e < 6; ++e) acc[((size_t)b * 32 + lane) * 6 + e] = 0.f;
+    for (int e = 0; e < 3; ++e) row[96 * b + e] = make_float2(0.f, 0.f);
   __syncwarp();
   const float d0[3] = {a.origin[0] - pose[0], a.origin[1] - pose[1], a.origin[2] - pose[2]};
   float Sl = 0.f, gs[3] = {0.f, 0.f, 0.f}, Gp[9];
@@ -408,41 +415,64 @@ __device__ float gl_eval(const GradArgs& a, const FkLigand& S, int N, int n, con
   float fa[6] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
   auto flush = [&]() {
     if (cur >= 0 && cur < n) {
-      float* ac = acc + ((size_t)cur * 32 + lane) * 6;
+      float2* ac = row + 96 * cur;
 #pragma unroll
-      for (int e = 0; e < 6; ++e) ac[e] += fa[e];
+      for (int e = 0; e < 3; ++e) {
+        const float2 v = ac[e];
+        ac[e] = make_float2(v.x + fa[2 * e], v.y + fa[2 * e + 1]);
+      }
     }
 #pragma unroll
     for (int e = 0; e < 6; ++e) fa[e] = 0.f;
   };
-  for (int i = sub; i < N; i += G) {
-    const float4 X = S.sx[i];
-    const int o = S.own[i];
-    if (o != cur) {
-      flush();
-      fk_get(T + ((size_t)o * PW + grp) * 12, m0, m1, m2);
-      cur = o;
+  int got = -1;   // the owner whose transform is in m0..m2
+  constexpr int A = GL<G>::kAhead;
+  for (int i0 = sub; i0 < N; i0 += G * A) {
+    FetchedRecord rec[A];
+    float u[A][3];
+    int own[A];
+#pragma unroll
+    for (int k = 0; k < A; ++k) {
+      const int i = min(i0 + k * G, N - 1);   // past the end: fetched, not added
+      const float4 X = S.sx[i];
+      own[k] = S.own[i];
+      if (own[k] != got) {
+        fk_get(T + ((size_t)own[k] * PW + grp) * 12, m0, m1, m2);
+        got = own[k];
+      }
+      u[k][0] = fmaf(m0.x, X.x, fmaf(m0.y, X.y, fmaf(m0.z, X.z, m0.w)));
+      u[k][1] = fmaf(m1.x, X.x, fmaf(m1.y, X.y, fmaf(m1.z, X.z, m1.w)));
+      u[k][2] = fmaf(m2.x, X.x, fmaf(m2.y, X.y, fmaf(m2.z, X.z, m2.w)));
+      rec[k] = grid_fetch(a.grid, u[k][0], u[k][1], u[k][2], __float_as_int(X.w));
     }
-    const float u[3] = {fmaf(m0.x, X.x, fmaf(m0.y, X.y, fmaf(m0.z, X.z, m0.w))),
-                        fmaf(m1.x, X.x, fmaf(m1.y, X.y, fmaf(m1.z, X.z, m1.w))),
-                        fmaf(m2.x, X.x, fmaf(m2.y, X.y, fmaf(m2.z, X.z, m2.w)))};
-    float gx, gy, gz;
-    Sl -= grid_sample_grad(a.grid, u[0], u[1], u[2], __float_as_int(X.w), &gx, &gy, &gz);
-    const float du[3] = {-gx, -gy, -gz};   // dS/du, per grid unit
 #pragma unroll
-    for (int r = 0; r < 3; ++r) gs[r] += du[r];
-    const float dv[3] = {fmaf(a.h, u[0], d0[0]), fmaf(a.h, u[1], d0[1]), fmaf(a.h, u[2], d0[2])};   // x - t, A
+    for (int k = 0; k < A; ++k) {
+      if (i0 + k * G >= N) break;
+      const int o = own[k];
+      if (o != cur) {
+        flush();
+        cur = o;
+      }
+      float gx, gy, gz;
+      Sl -= fetched_grad(a.grid, rec[k], &gx, &gy, &gz);
+      const float du[3] = {-gx, -gy, -gz};   // dS/du, per grid unit
 #pragma unroll
-    for (int r = 0; r < 3; ++r)
+      for (int r = 0; r < 3; ++r) gs[r] += du[r];
+      const float dv[3] = {fmaf(a.h, u[k][0], d0[0]), fmaf(a.h, u[k][1], d0[1]), fmaf(a.h, u[k][2], d0[2])};   // x - t, A
 #pragma unroll
-      for (int c = 0; c < 3; ++c) Gp[3 * r + c] = fmaf(du[r], dv[c], Gp[3 * r + c]);
-    if (o < n) {
-      fa[0] += du[0];
-      fa[1] += du[1];
-      fa[2] += du[2];
-      fa[3] += u[1] * du[2] - u[2] * du[1];
-      fa[4] += u[2] * du[0] - u[0] * du[2];
-      fa[5] += u[0] * du[1] - u[1] * du[0];
+      for (int r = 0; r < 3; ++r)
+#pragma unroll
+        for (int c = 0; c < 3; ++c) Gp[3 * r + c] = fmaf(du[r], dv[c], Gp[3 * r + c]);
+      if (o < n) {
+        fa[0] += du[0];
+        fa[1] += du[1];
+        fa[2] += du[2];
+        // u x du; which product is rounded first is part of the result (see
+        // the step norms below)
+        fa[3] = __fadd_rn(fa[3], fmaf(-u[k][2], du[1], __fmul_rn(u[k][1], du[2])));
+        fa[4] = __fadd_rn(fa[4], fmaf(-u[k][0], du[2], __fmul_rn(u[k][2], du[0])));
+        fa[5] = __fadd_rn(fa[5], fmaf(-u[k][1], du[0], __fmul_rn(u[k][0], du[1])));
+      }
     }
   }
   flush();
@@ -451,7 +481,10 @@ __device__ float gl_eval(const GradArgs& a, const FkLigand& S, int N, int n, con
     const int b = S.ord[r], pb = S.par[b];
     if (pb < n) {
 #pragma unroll
-      for (int e = 0; e < 6; ++e) acc[((size_t)pb * 32 + lane) * 6 + e] += acc[((size_t)b * 32 + lane) * 6 + e];
+      for (int e = 0; e < 3; ++e) {
+        const float2 v = row[96 * pb + e], w = row[96 * b + e];
+        row[96 * pb + e] = make_float2(v.x + w.x, v.y + w.y);
+      }
     }
   }
   Sl = gl_sum(Sl, G);
@@ -489,9 +522,10 @@ __device__ float gl_eval(const GradArgs& a, const FkLigand& S, int N, int n, con
   for (int b = sub; b < n; b += G) {   // torsion gradients, bonds over the group's lanes
     float F[3] = {0.f, 0.f, 0.f}, tau[3] = {0.f, 0.f, 0.f};
     for (int j = 0; j < G; ++j) {   // the group's lanes, in lane order
-      const float* ac = acc + ((size_t)b * 32 + grp * G + j) * 6;
-      F[0] += ac[0]; F[1] += ac[1]; F[2] += ac[2];
-      tau[0] += ac[3]; tau[1] += ac[4]; tau[2] += ac[5];
+      const float2* ac = reinterpret_cast<const float2*>(acc) + 96 * b + 3 * (grp * G + j);
+      const float2 v0 = ac[0], v1 = ac[1], v2 = ac[2];
+      F[0] += v0.x; F[1] += v0.y; F[2] += v1.x;
+      tau[0] += v1.y; tau[1] += v2.x; tau[2] += v2.y;
     }
     float4 p0, p1, p2;
     fk_get(T + ((size_t)S.par[b] * PW + grp) * 12, p0, p1, p2);
@@ -561,46 +595,52 @@ __global__ void __launch_bounds__(32, 16) grad_lane_kernel(const GradArgs a) {
   } else {
     float s_t = a.step_t, s_q = a.step_q, s_th = a.step_theta;
     for (int s = 0; s < a.steps; ++s) {
-      if (sub == 0) {
-        float nt = 0.f, nq = 0.f, nth = 0.f;
-        for (int e = 0; e < plen; ++e) {
-          const float v = grad[e] * grad[e];
-          if (e < 3) nt += v; else if (e < 7) nq += v; else nth += v;
-        }
-        nt = sqrtf(nt); nq = sqrtf(nq); nth = sqrtf(nth);
-        const float kt = nt > 0.f ? s_t / nt : 0.f;
-        const float kq = nq > 0.f ? s_q / nq : 0.f;
-        const float kth = nth > 0.f ? s_th / nth : 0.f;
-        const float rqn = 1.f / sqrtf(pose[3] * pose[3] + pose[4] * pose[4] + pose[5] * pose[5] + pose[6] * pose[6]);
-        float qq[4], qm = 0.f;
+      // Every lane of the group takes the norms and step factors (the same
+      // instructions as one lane doing it); the angles go round-robin. Which
+      // squares are fused into their sum is fixed: a refined pose follows
+      // from comparisons of scores, so an ulp here can part two trajectories.
+      float nt = 0.f, nq = 0.f, nth = 0.f;
 #pragma unroll
-        for (int k = 0; k < 4; ++k) {
-          qq[k] = fmaf(kq, grad[3 + k], pose[3 + k] * rqn);
-          qm += qq[k] * qq[k];
+      for (int e = 0; e < 3; ++e) nt = __fadd_rn(nt, __fmul_rn(grad[e], grad[e]));
+#pragma unroll
+      for (int e = 3; e < 7; ++e) nq = __fadd_rn(nq, __fmul_rn(grad[e], grad[e]));
+      const int whole = plen & ~3;
+#pragma unroll 4
+      for (int e = 7; e < plen; ++e) {
+        const float v = grad[e];
+        nth = (e & 3) == 3 && e < whole ? fmaf(v, v, nth) : __fadd_rn(nth, __fmul_rn(v, v));
+      }
+      nt = sqrtf(nt); nq = sqrtf(nq); nth = sqrtf(nth);
+      const float kt = nt > 0.f ? s_t / nt : 0.f;
+      const float kq = nq > 0.f ? s_q / nq : 0.f;
+      const float kth = nth > 0.f ? s_th / nth : 0.f;
+      const float rqn = 1.f / sqrtf(pose[3] * pose[3] + pose[4] * pose[4] + pose[5] * pose[5] + pose[6] * pose[6]);
+      float qq[4], qm = 0.f;
+#pragma unroll
+      for (int k = 0; k < 4; ++k) {
+        qq[k] = fmaf(kq, grad[3 + k], pose[3 + k] * rqn);
+        qm = fmaf(qq[k], qq[k], qm);
+      }
+      const float rqm = 1.f / sqrtf(qm);
+      if (sub == 0) {
+#pragma unroll
+        for (int e = 0; e < 3; ++e)
+          cand[e] = fminf(fmaxf(fmaf(kt, grad[e], pose[e]), a.box_lo[e]), a.box_hi[e]);
+#pragma unroll
+        for (int k = 0; k < 4; ++k) cand[3 + k] = qq[k] * rqm;
+      }
+      for (int e = 7 + sub; e < plen; e += G) {
+        // wrap to [-pi, pi): one turn suffices from a wrapped angle;
+        // other inputs take the general reduction
+        const float w0 = fmaf(kth, grad[e], pose[e]) + kPiF;
+        float w = w0;
+        if (w >= 2.f * kPiF) w -= 2.f * kPiF;
+        else if (w < 0.f) w += 2.f * kPiF;
+        if (!(w >= 0.f && w < 2.f * kPiF)) {
+          w = fmodf(w0, 2.f * kPiF);
+          if (w < 0.f) w += 2.f * kPiF;
         }
-        const float rqm = 1.f / sqrtf(qm);
-        for (int e = 0; e < plen; ++e) {
-          float v;
-          if (e < 3) {
-            v = fmaf(kt, grad[e], pose[e]);
-            v = fminf(fmaxf(v, a.box_lo[e]), a.box_hi[e]);
-          } else if (e < 7) {
-            v = qq[e - 3] * rqm;
-          } else {
-            // wrap to [-pi, pi): one turn suffices from a wrapped angle;
-            // other inputs take the general reduction
-            const float w0 = fmaf(kth, grad[e], pose[e]) + kPiF;
-            float w = w0;
-            if (w >= 2.f * kPiF) w -= 2.f * kPiF;
-            else if (w < 0.f) w += 2.f * kPiF;
-            if (!(w >= 0.f && w < 2.f * kPiF)) {
-              w = fmodf(w0, 2.f * kPiF);
-              if (w < 0.f) w += 2.f * kPiF;
-            }
-            v = w - kPiF;
-          }
-          cand[e] = v;
-        }
+        cand[e] = w - kPiF;
       }
       __syncwarp();
       // the candidate with its gradient: a kept step needs no second evaluation

@@ -98,7 +98,7 @@ __device__ __forceinline__ double trilinear64(const RescoreArgs& a, const Tri64&
 // every (pose, bond) [pose][bond][2].
 __host__ __device__ inline size_t rs_warp_bytes(int acap, int ncap, unsigned char* base, FkLigand* S, double** B,
                                                 double** T, double** Y, double** SC) {
-  const size_t lb = fk_ligand_carve(acap, ncap, base, S);   // a multiple of 16
+  const size_t lb = fk_ligand_carve(acap, ncap, base, S, true);   // a multiple of 16
   const size_t bb = (size_t)ncap * 6 * sizeof(double);
   const size_t tb = (size_t)(ncap + 1) * kRsPoses * 12 * sizeof(double);
   const size_t yb = ((size_t)acap * 3 * sizeof(double) + 15) & ~(size_t)15;

@@ -103,7 +103,7 @@ template <int G>
 __host__ __device__ inline size_t lane_carve(int acap, int ncap, unsigned char* base, FkLigand* S, float** T) {
   const size_t tbytes = (size_t)(ncap + 1) * (32 / G) * 12 * sizeof(float);
   if (T) *T = (float*)base;
-  return tbytes + fk_ligand_carve(acap, ncap, base ? base + tbytes : nullptr, S);
+  return tbytes + fk_ligand_carve(acap, ncap, base ? base + tbytes : nullptr, S, false);
 }
 
 // Work item gw = (ligand entry, 32/G poses) of the warp.
