@@ -114,6 +114,19 @@ __device__ __forceinline__ void torsion_cs(int j, int step_deg, float* c, float*
   sincospif((float)(j * step_deg) * (1.0f / 180.0f), s, c);
 }
 
+// The angle of torsion increment j as poses hold it: radians in [-pi, pi).
+__device__ __forceinline__ float torsion_radians(int j, int step_deg) {
+  int deg = (j * step_deg) % 360;
+  if (deg >= 180) deg -= 360;
+  return (float)deg * 0.017453292519943295f;
+}
+
+// The increment of an angle written by torsion_radians.
+__device__ __forceinline__ int torsion_increment(float radians, int step_deg, int n_theta) {
+  const int j = __float2int_rn(radians * 57.29577951308232f / (float)step_deg);
+  return j < 0 ? j + n_theta : j;
+}
+
 // Rotation of point x by the angle with cosine c and sine s about the line
 // through v with unit direction k (right-handed): the component along k
 // stays, the perpendicular part turns. Same arithmetic as the docking

@@ -16,9 +16,9 @@
 // coordinates, the bond records and moving-atom lists (coalesced loads);
 // each atom's owner; each bond's parent (the owner of its moving endpoint v,
 // which no other bond's list holds); the bonds in decreasing moving-side
-// size (a parent before its children) and grouped by depth in the bond
-// tree; the bond axes. The packer writes the same values out once per ligand
-// (the table, with the atoms listed by owner); the scoring and gradient
+// size (a parent before its children); the bond axes. The packer writes the
+// same values, and the bonds grouped by depth in the bond tree, out once per
+// ligand (the table, with the atoms listed by owner); the scoring and gradient
 // kernels stage it with fk_load (vector copies). Transforms are 12 floats:
 // three rows (m0 m1 m2 | o).
 #pragma once
@@ -81,11 +81,9 @@ __host__ __device__ inline size_t fk_ligand_carve(int acap, int ncap, unsigned c
   return o;
 }
 
-// Stage ligand (a0, N, r0, n) for the warp (all 32 lanes call it); DEPTHS:
-// also the bonds grouped by depth (lord, loff) for fk_transforms_group.
-// Returns false, on every lane, when a bond endpoint or a moving atom is out
+// Stage ligand (a0, N, r0, n) for the warp (all 32 lanes call it), without
+// the bonds' grouping by depth. Returns false, on every lane, when a bond endpoint or a moving atom is out
 // of range (nothing out of range is written).
-template <bool DEPTHS = false>
 __device__ inline bool fk_stage(const Packed& pk, int a0, int N, int r0, int n, const FkLigand& S, int lane) {
   for (int i = lane; i < N; i += 32) {
     S.sx[i] = pk.xc[a0 + i];
@@ -132,34 +130,14 @@ __device__ inline bool fk_stage(const Packed& pk, int a0, int N, int r0, int n, 
   }
   bad = __any_sync(0xffffffffu, bad);
   __syncwarp();
-  if (DEPTHS && lane == 0 && !bad) {   // depths (parents first in ord), then bonds by depth
-    uint8_t depth[LIGEN_MAX_ROT];
-    int cnt[LIGEN_MAX_ROT + 1] = {};
-    int dmax = -1;
-    for (int r = 0; r < n; ++r) {
-      const int b = S.ord[r], pb = S.par[b];
-      depth[b] = (uint8_t)(pb == n ? 0 : depth[pb] + 1);
-      ++cnt[depth[b]];
-      dmax = depth[b] > dmax ? depth[b] : dmax;
-    }
-    int o = 0;
-    for (int d = 0; d <= dmax; ++d) {
-      S.loff[d] = (uint8_t)o;
-      o += cnt[d];
-    }
-    S.loff[dmax + 1] = (uint8_t)n;
-    for (int d = 0; d <= dmax; ++d) cnt[d] = S.loff[d];
-    for (int r = 0; r < n; ++r) S.lord[cnt[depth[S.ord[r]]]++] = S.ord[r];
-    S.loff[LIGEN_MAX_ROT] = (uint8_t)(dmax + 1);   // number of depths
-  }
   __syncwarp();
   return !bad;
 }
 
 // Stage ligand l = (a0, N, r0, n) for the warp (all 32 lanes call it) from
 // the forward-kinematics table (pk.fk_*, written by the packer): the
-// contents fk_stage<true> builds, but for the moving-atom lists (nothing
-// reads them after staging), with the atoms listed by owner (S.sx, S.own in
+// contents fk_stage builds, but for the moving-atom lists (nothing reads
+// them after staging), and the bonds grouped by depth, with the atoms listed by owner (S.sx, S.own in
 // the table's order) and S.sb[b].y the list position of bond b's v (S.sb[b].x
 // unused). Vector copies, no per-bond passes. Returns false, on every lane, when the table marks the ligand's
 // lists as malformed.

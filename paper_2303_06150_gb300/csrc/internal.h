@@ -148,13 +148,17 @@ struct RescoreArgs {
   int K;                    // kept poses per ligand
   int max_atoms;            // largest ligand (shared-memory carve-up)
   int max_rot;              // most rotatable bonds of a ligand (shared-memory carve-up)
-  float* poses;             // outputs, re-ranked in place
+  double inv_h;             // 1 / h
+  int step_deg, n_theta;    // torsions are whole increments of step_deg degrees
+  bool small_axes;          // no axis has more than 2^20 points
+  const float* poses;       // the kept poses and their restarts, in FP32 order
+  const int32_t* tmp_top;
+  float* out_poses;         // outputs, re-ranked
   float* scores;            // [L][K], FP64 scores rounded to FP32
   int32_t* top_restart;     // [L][K] or NULL
-  double* out_s64;          // [L][K] or NULL: FP64 scores, re-ranked
+  double* out_s64;          // [L][K] or NULL: FP64 scores
   double* s64;              // scratch [L][K]
-  const float* tmp_poses;   // copy of the poses before re-ranking
-  const int32_t* tmp_top;   // copy of top_restart before re-ranking, or NULL
+  double* table;            // scratch [n_theta][2]
   unsigned* check;          // checked builds: first out-of-range code, else NULL
 };
 

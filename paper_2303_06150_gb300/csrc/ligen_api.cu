@@ -960,12 +960,15 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     if (params->top_restart) o_top = ar.take(4 * (size_t)L * K);
   }
   const bool rescore = params->rescore_fp64 == 1;
-  size_t o_itop = 0, o_tmp_poses = 0, o_tmp_top = 0, o_s64 = 0, o_out64 = 0;
-  if (rescore) {
-    if (!params->top_restart) o_itop = ar.take(4 * (size_t)L * K);   // restart ids for tie-breaks
+  size_t o_tmp_poses = 0, o_tmp_top = 0, o_s64 = 0, o_table = 0, o_out64 = 0;
+  if (rescore) {   // top-K writes here, the re-rank to the outputs
     o_tmp_poses = ar.take(4 * pose_floats);
     o_tmp_top = ar.take(4 * (size_t)L * K);
     o_s64 = ar.take(8 * (size_t)L * K);
+    // the increments' sines and cosines: over the grid records, which nothing
+    // reads after docking, where those are larger
+    const size_t need = 16 * (size_t)(360 / params->torsion_step_deg);
+    o_table = coef_max >= need ? o_coef : ar.take(need);
     if (params->scores_f64 && ohost) o_out64 = ar.take(8 * (size_t)L * K);
   }
   const bool buckets = params->batching != LIGEN_BATCH_PLAIN && !exhaustive;
@@ -1060,7 +1063,6 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     int16_t* d_trace = site_trace ? (ohost ? ar.at<int16_t>(o_trace) : site_trace) : nullptr;
     float* d_coords = site_coords ? (ohost ? ar.at<float>(o_coords) : site_coords) : nullptr;
     int32_t* d_top = site_top ? (ohost ? ar.at<int32_t>(o_top) : site_top) : nullptr;
-    if (rescore && !d_top) d_top = ar.at<int32_t>(o_itop);
 
     DockArgs da{};
     da.lig = lig;
@@ -1126,15 +1128,13 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     ta.seed = params->seed;
     for (int k = 0; k < 3; ++k) ta.center[k] = da.center[k];
     ta.jitter = params->jitter;
-    ta.out_poses = d_poses;
+    ta.out_poses = rescore ? ar.at<float>(o_tmp_poses) : d_poses;
     ta.out_scores = d_scores;
-    ta.top_restart = d_top;
+    ta.top_restart = rescore ? ar.at<int32_t>(o_tmp_top) : d_top;   // re-ranking breaks ties by restart
     LG_CUDA(launch_topk(ta, s));
     double* d_out64 = nullptr;
     if (rescore) {
       d_out64 = site_s64 ? (ohost ? ar.at<double>(o_out64) : site_s64) : nullptr;
-      LG_CUDA(cudaMemcpyAsync(ar.base + o_tmp_poses, d_poses, 4 * pose_floats, cudaMemcpyDeviceToDevice, s));
-      LG_CUDA(cudaMemcpyAsync(ar.base + o_tmp_top, d_top, 4 * (size_t)L * K, cudaMemcpyDeviceToDevice, s));
       RescoreArgs rsa{};
       rsa.lig = lig;
       rsa.pk = pk;
@@ -1147,12 +1147,17 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
       rsa.K = K;
       rsa.max_atoms = sh.max_atoms;
       rsa.max_rot = sh.max_rot;
-      rsa.poses = d_poses;
+      rsa.inv_h = 1.0 / rsa.h;
+      rsa.step_deg = params->torsion_step_deg;
+      rsa.n_theta = 360 / params->torsion_step_deg;
+      rsa.small_axes = std::max({grid->nx, grid->ny, grid->nz}) <= 1 << 20;
+      rsa.out_poses = d_poses;
       rsa.scores = d_scores;
-      rsa.top_restart = site_top ? d_top : nullptr;
+      rsa.top_restart = d_top;
       rsa.out_s64 = d_out64;
       rsa.s64 = ar.at<double>(o_s64);
-      rsa.tmp_poses = ar.at<float>(o_tmp_poses);
+      rsa.table = ar.at<double>(o_table);
+      rsa.poses = ar.at<float>(o_tmp_poses);
       rsa.tmp_top = ar.at<int32_t>(o_tmp_top);
       rsa.check = chk.d;
       LG_CUDA(launch_rescore(rsa, s));
