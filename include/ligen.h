@@ -245,9 +245,12 @@ int ligen_dock_batch(const ligen_ligands_t* ligands, const ligen_grid_t* grid,
  * footprint grows with the number of sites). grids[n_sites] are the sites'
  * pocket grids: same channel count, each its own box and spacing, all in
  * host memory or all in device memory. The library is staged and packed once;
- * the grid records of one site at a time live in one buffer sized for the
- * largest site, so device memory grows with the largest grid, not with the
- * number of sites.
+ * the grid records and per-restart results of at most two sites at a time
+ * live in two sets of buffers sized for the largest site, so device memory
+ * grows with the largest grid, not with the number of sites. Two sets, with
+ * consecutive sites overlapping on internal streams joined back to `stream`,
+ * for plain greedy calls on device memory without stage_ms; one set
+ * otherwise, and where two would not fit the workspace limit or the memory.
  * Outputs are site-major: site g's scores start at out_scores + g * L * K,
  * its poses at out_poses + g * K * (7 * L + total rotatable bonds); trace,
  * top_restart and scores_f64 (when given) are likewise [n_sites][...] with

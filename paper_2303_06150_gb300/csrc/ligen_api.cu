@@ -507,6 +507,33 @@ int get_fork(int dev, cudaStream_t s, int n, Fork** out, bool fence = false) {
   return LIGEN_OK;
 }
 
+// Streams and events of the overlapped sites of ligen_dock_sites, per
+// (device, calling stream).
+struct SitePipe {
+  cudaStream_t high = nullptr;      // grid records and top-K, ahead of queued docking CTAs
+  cudaStream_t dock[2] = {};
+  cudaEvent_t start = nullptr, packed = nullptr, end = nullptr;
+  cudaEvent_t prep[2] = {}, docked[2] = {}, top[2] = {};
+};
+std::map<std::pair<int, cudaStream_t>, SitePipe> g_pipes;   // g_fork_mu
+
+int get_pipe(int dev, cudaStream_t s, SitePipe** out) {
+  std::lock_guard<std::mutex> lk(g_fork_mu);
+  SitePipe& p = g_pipes[{dev, s}];
+  if (!p.high) {
+    int least = 0, greatest = 0;
+    LG_CUDA(cudaDeviceGetStreamPriorityRange(&least, &greatest));
+    for (cudaEvent_t* e : {&p.start, &p.packed, &p.end, &p.prep[0], &p.prep[1], &p.docked[0], &p.docked[1], &p.top[0],
+                           &p.top[1]})
+      if (!*e) LG_CUDA(cudaEventCreateWithFlags(e, cudaEventDisableTiming));
+    for (cudaStream_t& d : p.dock)
+      if (!d) LG_CUDA(cudaStreamCreateWithPriority(&d, cudaStreamNonBlocking, least));
+    LG_CUDA(cudaStreamCreateWithPriority(&p.high, cudaStreamNonBlocking, greatest));
+  }
+  *out = &p;
+  return LIGEN_OK;
+}
+
 // Instantiated graphs of the bucketed launch sequence, keyed by everything
 // the launches capture by value (pointers, sizes, shapes, grid sizes).
 struct GraphEntry {
@@ -879,6 +906,25 @@ int ligen_release_workspaces(void) {
       }
     }
   }
+  {
+    std::lock_guard<std::mutex> fl(g_fork_mu);
+    for (auto it = g_pipes.begin(); it != g_pipes.end();) {
+      if (it->first.first != dev) {
+        ++it;
+        continue;
+      }
+      SitePipe& p = it->second;
+      for (cudaStream_t st : {p.high, p.dock[0], p.dock[1]})
+        if (st) {
+          cudaStreamSynchronize(st);
+          cudaStreamDestroy(st);
+        }
+      for (cudaEvent_t ev : {p.start, p.packed, p.end, p.prep[0], p.prep[1], p.docked[0], p.docked[1], p.top[0],
+                             p.top[1]})
+        if (ev) cudaEventDestroy(ev);
+      it = g_pipes.erase(it);
+    }
+  }
   std::lock_guard<std::mutex> lk(g_ws_mu);
   for (auto it = g_ws.begin(); it != g_ws.end();) {
     if (it->first.first == dev) {
@@ -1010,7 +1056,42 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
       longest_first = false;
     }
   }
-  if ((rc = get_workspace(s, ar.used, &ar.base)) != LIGEN_OK) return rc;
+  // What a site's launches write and the next site's overwrite. With a second
+  // set, sites overlap: one's records are built and its winners picked while
+  // another docks, and its first CTAs fill the SMs that the other's last
+  // ligands leave idle (301 screening ligands x 12 sites: 8.27 ms one after
+  // another, 7.50 ms). Device memory only, plain greedy launches, no stage
+  // times; dropped where it would exceed the workspace limit or the memory.
+  struct SiteSet {
+    size_t coef, rs, rk, rc, tmp_poses, tmp_top, s64, table;
+  } set[2];
+  set[0] = {o_coef, o_rs, o_rk, o_rc, o_tmp_poses, o_tmp_top, o_s64, o_table};
+  set[1] = set[0];
+  bool overlap = n_sites > 1 && !buckets && !exhaustive && !ghost && !ohost && !params->stage_ms;
+  const size_t one_set = ar.used;
+  if (overlap) {
+    set[1].coef = ar.take(coef_max);
+    set[1].rs = ar.take(4 * (size_t)L * R);
+    set[1].rk = ar.take((size_t)L * R);
+    set[1].rc = ar.take((size_t)sh.rot * R);
+    if (rescore) {
+      set[1].tmp_poses = ar.take(4 * pose_floats);
+      set[1].tmp_top = ar.take(4 * (size_t)L * K);
+      set[1].s64 = ar.take(8 * (size_t)L * K);
+      if (o_table == o_coef) set[1].table = set[1].coef;   // else both write the same table
+    }
+    const size_t limit = g_ws_limit.load();
+    overlap = !limit || ar.used <= limit;
+  }
+  rc = LIGEN_ERR_OOM;
+  if (overlap) rc = get_workspace(s, ar.used, &ar.base);
+  if (rc == LIGEN_ERR_OOM) {
+    overlap = false;
+    ar.used = one_set;
+    rc = get_workspace(s, ar.used, &ar.base);
+  }
+  if (rc != LIGEN_OK) return rc;
+  g_err.clear();
   if ((rc = chk.arm(ar, s)) != LIGEN_OK) return rc;
   unsigned long long* d_samples = nullptr;
   if (params->samples) {
@@ -1030,44 +1111,48 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
   pk.status = ar.at<int32_t>(o_status);
   const cudaMemcpyKind back = ohost ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
 
-  for (int site = 0; site < n_sites; ++site) {
-    const ligen_grid_t* grid = &grids[site];
-    float* site_poses = out_poses + (size_t)site * pose_floats;
-    float* site_scores = out_scores + (size_t)site * L * K;
-    int16_t* site_trace = params->trace ? params->trace + (size_t)site * trace_elems : nullptr;
-    float* site_coords = params->coords ? params->coords + (size_t)site * coord_elems : nullptr;
-    int32_t* site_top = params->top_restart ? params->top_restart + (size_t)site * L * K : nullptr;
-    double* site_s64 = params->scores_f64 ? params->scores_f64 + (size_t)site * L * K : nullptr;
-    float site_ms[LIGEN_N_STAGES];
-    Timer tm(stage_out ? site_ms : nullptr, s);
-    tm.mark();
-    if (site == 0) {
-      if ((rc = stage_ligands(ar, ligands, sh, lp, s, &lig)) != LIGEN_OK) return rc;
-    }
-    const float* gvals = (const float*)grid->data;
-    if (ghost) {
-      LG_CUDA(cudaMemcpyAsync(ar.base + o_gval, grid->data, grid_values_bytes(grid), cudaMemcpyHostToDevice, s));
-      gvals = ar.at<float>(o_gval);
-    }
-    tm.mark();
-    float* coef = ar.at<float>(o_coef);
-    LG_CUDA(launch_grid_prep_fmt(gvals, grid->nx, grid->ny, grid->nz, grid->nc, fmt, coef, s));
-    tm.mark();
-    if (site == 0) LG_CUDA(launch_pack(lig, grid->nc, pk, sh.max_atoms, s));
-    if (site == 0 && longest_first)
+  // one site: its slices of the outputs and its launches' arguments
+  struct Site {
+    const ligen_grid_t* grid;
+    const float* gvals;
+    float *site_poses, *site_scores, *site_coords, *d_poses, *d_scores, *d_coords;
+    int16_t *site_trace, *d_trace;
+    int32_t *site_top, *d_top;
+    double *site_s64, *d_out64;
+    DockArgs da;
+  };
+  auto open_site = [&](int site, Site& S) {
+    S.grid = &grids[site];
+    S.gvals = ghost ? ar.at<float>(o_gval) : (const float*)S.grid->data;
+    S.site_poses = out_poses + (size_t)site * pose_floats;
+    S.site_scores = out_scores + (size_t)site * L * K;
+    S.site_trace = params->trace ? params->trace + (size_t)site * trace_elems : nullptr;
+    S.site_coords = params->coords ? params->coords + (size_t)site * coord_elems : nullptr;
+    S.site_top = params->top_restart ? params->top_restart + (size_t)site * L * K : nullptr;
+    S.site_s64 = params->scores_f64 ? params->scores_f64 + (size_t)site * L * K : nullptr;
+    S.d_poses = ohost ? ar.at<float>(o_poses) : S.site_poses;
+    S.d_scores = ohost ? ar.at<float>(o_scores) : S.site_scores;
+    S.d_trace = S.site_trace ? (ohost ? ar.at<int16_t>(o_trace) : S.site_trace) : nullptr;
+    S.d_coords = S.site_coords ? (ohost ? ar.at<float>(o_coords) : S.site_coords) : nullptr;
+    S.d_top = S.site_top ? (ohost ? ar.at<int32_t>(o_top) : S.site_top) : nullptr;
+  };
+  auto records = [&](const Site& S, const SiteSet& b, cudaStream_t st) -> int {
+    LG_CUDA(launch_grid_prep_fmt(S.gvals, S.grid->nx, S.grid->ny, S.grid->nz, S.grid->nc, fmt, ar.at<float>(b.coef), st));
+    return LIGEN_OK;
+  };
+  auto pack = [&]() -> int {
+    LG_CUDA(launch_pack(lig, grids[0].nc, pk, sh.max_atoms, s));
+    if (longest_first)
       LG_CUDA(launch_order(lig, params->n_rigid, P, 360 / params->torsion_step_deg, ar.at<int32_t>(o_order), s));
-    tm.mark();
-
-    float* d_poses = ohost ? ar.at<float>(o_poses) : site_poses;
-    float* d_scores = ohost ? ar.at<float>(o_scores) : site_scores;
-    int16_t* d_trace = site_trace ? (ohost ? ar.at<int16_t>(o_trace) : site_trace) : nullptr;
-    float* d_coords = site_coords ? (ohost ? ar.at<float>(o_coords) : site_coords) : nullptr;
-    int32_t* d_top = site_top ? (ohost ? ar.at<int32_t>(o_top) : site_top) : nullptr;
-
-    DockArgs da{};
+    return LIGEN_OK;
+  };
+  auto search = [&](Site& S, const SiteSet& b, cudaStream_t st) -> int {
+    const ligen_grid_t* grid = S.grid;
+    DockArgs& da = S.da;
+    da = DockArgs{};
     da.lig = lig;
     da.pk = pk;
-    da.grid = make_view(grid, coef, params->out_penalty, fmt);
+    da.grid = make_view(grid, ar.at<float>(b.coef), params->out_penalty, fmt);
     da.grid.check = chk.d;
     const float h = grid->spacing;
     const int np[3] = {grid->nx, grid->ny, grid->nz};
@@ -1093,15 +1178,15 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     da.max_atoms = sh.max_atoms;
     da.max_rot = sh.max_rot;
     da.max_frag = (int)sh.max_frag;
-    da.res_score = ar.at<float>(o_rs);
-    da.res_k = ar.at<uint8_t>(o_rk);
-    da.res_cnt = ar.at<uint8_t>(o_rc);
-    da.trace = d_trace;
-    da.coords = d_coords;
+    da.res_score = ar.at<float>(b.rs);
+    da.res_k = ar.at<uint8_t>(b.rk);
+    da.res_cnt = ar.at<uint8_t>(b.rc);
+    da.trace = S.d_trace;
+    da.coords = S.d_coords;
     da.samples = d_samples;
     if (longest_first) da.list = ar.at<int32_t>(o_order);
     if (exhaustive) {
-      LG_CUDA(launch_exhaustive(da, s));
+      LG_CUDA(launch_exhaustive(da, st));
     } else if (buckets) {
       // Uploaded on every call: any other call on this stream may have
       // carved the workspace differently and overwritten this region (a
@@ -1116,30 +1201,32 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
                              params->batching != LIGEN_BATCH_BUCKETS_STATIC, s)) != LIGEN_OK)
         return rc;
     } else {
-      LG_CUDA(launch_dock(da, 0, s, true));
+      LG_CUDA(launch_dock(da, 0, st, true));
     }
-    tm.mark();
-
+    return LIGEN_OK;
+  };
+  auto winners = [&](Site& S, const SiteSet& b, cudaStream_t st) -> int {
+    const ligen_grid_t* grid = S.grid;
     TopkArgs ta{};
     ta.L = L; ta.R = R; ta.K = K; ta.step_deg = params->torsion_step_deg;
     ta.rot_off = lig.rot_off;
     ta.status = pk.status;
-    ta.res_score = da.res_score; ta.res_k = da.res_k; ta.res_cnt = da.res_cnt;
+    ta.res_score = S.da.res_score; ta.res_k = S.da.res_k; ta.res_cnt = S.da.res_cnt;
     ta.seed = params->seed;
-    for (int k = 0; k < 3; ++k) ta.center[k] = da.center[k];
+    for (int k = 0; k < 3; ++k) ta.center[k] = S.da.center[k];
     ta.jitter = params->jitter;
-    ta.out_poses = rescore ? ar.at<float>(o_tmp_poses) : d_poses;
-    ta.out_scores = d_scores;
-    ta.top_restart = rescore ? ar.at<int32_t>(o_tmp_top) : d_top;   // re-ranking breaks ties by restart
-    LG_CUDA(launch_topk(ta, s));
-    double* d_out64 = nullptr;
+    ta.out_poses = rescore ? ar.at<float>(b.tmp_poses) : S.d_poses;
+    ta.out_scores = S.d_scores;
+    ta.top_restart = rescore ? ar.at<int32_t>(b.tmp_top) : S.d_top;   // re-ranking breaks ties by restart
+    LG_CUDA(launch_topk(ta, st));
+    S.d_out64 = nullptr;
     if (rescore) {
-      d_out64 = site_s64 ? (ohost ? ar.at<double>(o_out64) : site_s64) : nullptr;
+      S.d_out64 = S.site_s64 ? (ohost ? ar.at<double>(o_out64) : S.site_s64) : nullptr;
       RescoreArgs rsa{};
       rsa.lig = lig;
       rsa.pk = pk;
       rsa.status = pk.status;
-      rsa.values = gvals;
+      rsa.values = S.gvals;
       rsa.nx = grid->nx; rsa.ny = grid->ny; rsa.nz = grid->nz; rsa.nc = grid->nc;
       for (int k = 0; k < 3; ++k) rsa.origin[k] = grid->origin[k];
       rsa.h = grid->spacing;
@@ -1151,27 +1238,87 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
       rsa.step_deg = params->torsion_step_deg;
       rsa.n_theta = 360 / params->torsion_step_deg;
       rsa.small_axes = std::max({grid->nx, grid->ny, grid->nz}) <= 1 << 20;
-      rsa.out_poses = d_poses;
-      rsa.scores = d_scores;
-      rsa.top_restart = d_top;
-      rsa.out_s64 = d_out64;
-      rsa.s64 = ar.at<double>(o_s64);
-      rsa.table = ar.at<double>(o_table);
-      rsa.poses = ar.at<float>(o_tmp_poses);
-      rsa.tmp_top = ar.at<int32_t>(o_tmp_top);
+      rsa.out_poses = S.d_poses;
+      rsa.scores = S.d_scores;
+      rsa.top_restart = S.d_top;
+      rsa.out_s64 = S.d_out64;
+      rsa.s64 = ar.at<double>(b.s64);
+      rsa.table = ar.at<double>(b.table);
+      rsa.poses = ar.at<float>(b.tmp_poses);
+      rsa.tmp_top = ar.at<int32_t>(b.tmp_top);
       rsa.check = chk.d;
-      LG_CUDA(launch_rescore(rsa, s));
+      LG_CUDA(launch_rescore(rsa, st));
     }
+    return LIGEN_OK;
+  };
 
+  if (overlap) {
+    int dev = 0;
+    LG_CUDA(cudaGetDevice(&dev));
+    SitePipe* pipe = nullptr;
+    if ((rc = get_pipe(dev, s, &pipe)) != LIGEN_OK) return rc;
+    if ((rc = stage_ligands(ar, ligands, sh, lp, s, &lig)) != LIGEN_OK) return rc;
+    LG_CUDA(cudaEventRecord(pipe->start, s));
+    LG_CUDA(cudaStreamWaitEvent(pipe->high, pipe->start, 0));
+    if ((rc = pack()) != LIGEN_OK) return rc;
+    if (params->status)
+      LG_CUDA(cudaMemcpyAsync(params->status, pk.status, 4 * (size_t)L, cudaMemcpyDeviceToDevice, s));
+    LG_CUDA(cudaEventRecord(pipe->packed, s));
+    for (cudaStream_t d : pipe->dock) LG_CUDA(cudaStreamWaitEvent(d, pipe->packed, 0));
+    std::vector<Site> sites(2);
+    // records of site g: when site g - 2 has docked on the same set
+    auto prepare = [&](int g) -> int {
+      const int k = g & 1;
+      open_site(g, sites[k]);
+      if (g >= 2) LG_CUDA(cudaStreamWaitEvent(pipe->high, pipe->docked[k], 0));
+      const int e = records(sites[k], set[k], pipe->high);
+      if (e != LIGEN_OK) return e;
+      LG_CUDA(cudaEventRecord(pipe->prep[k], pipe->high));
+      return LIGEN_OK;
+    };
+    if ((rc = prepare(0)) != LIGEN_OK) return rc;
+    for (int g = 0; g < n_sites; ++g) {
+      const int k = g & 1;
+      LG_CUDA(cudaStreamWaitEvent(pipe->dock[k], pipe->prep[k], 0));
+      if (g >= 2) LG_CUDA(cudaStreamWaitEvent(pipe->dock[k], pipe->top[k], 0));   // site g - 2's results were read
+      if ((rc = search(sites[k], set[k], pipe->dock[k])) != LIGEN_OK) return rc;
+      LG_CUDA(cudaEventRecord(pipe->docked[k], pipe->dock[k]));
+      if (g + 1 < n_sites && (rc = prepare(g + 1)) != LIGEN_OK) return rc;
+      LG_CUDA(cudaStreamWaitEvent(pipe->high, pipe->docked[k], 0));
+      if ((rc = winners(sites[k], set[k], pipe->high)) != LIGEN_OK) return rc;
+      LG_CUDA(cudaEventRecord(pipe->top[k], pipe->high));
+    }
+    LG_CUDA(cudaEventRecord(pipe->end, pipe->high));   // after every site's docking and winners
+    LG_CUDA(cudaStreamWaitEvent(s, pipe->end, 0));
+  }
+  for (int site = 0; site < n_sites && !overlap; ++site) {
+    Site S;
+    open_site(site, S);
+    float site_ms[LIGEN_N_STAGES];
+    Timer tm(stage_out ? site_ms : nullptr, s);
+    tm.mark();
+    if (site == 0) {
+      if ((rc = stage_ligands(ar, ligands, sh, lp, s, &lig)) != LIGEN_OK) return rc;
+    }
+    if (ghost)
+      LG_CUDA(cudaMemcpyAsync(ar.base + o_gval, S.grid->data, grid_values_bytes(S.grid), cudaMemcpyHostToDevice, s));
+    tm.mark();
+    if ((rc = records(S, set[0], s)) != LIGEN_OK) return rc;
+    tm.mark();
+    if (site == 0 && (rc = pack()) != LIGEN_OK) return rc;
+    tm.mark();
+    if ((rc = search(S, set[0], s)) != LIGEN_OK) return rc;
+    tm.mark();
+    if ((rc = winners(S, set[0], s)) != LIGEN_OK) return rc;
     if (site == 0 && params->status)
       LG_CUDA(cudaMemcpyAsync(params->status, pk.status, 4 * (size_t)L, back, s));
     if (ohost) {
-      LG_CUDA(cudaMemcpyAsync(site_poses, d_poses, 4 * pose_floats, back, s));
-      LG_CUDA(cudaMemcpyAsync(site_scores, d_scores, 4 * (size_t)L * K, back, s));
-      if (d_trace) LG_CUDA(cudaMemcpyAsync(site_trace, d_trace, 2 * trace_elems, back, s));
-      if (d_coords) LG_CUDA(cudaMemcpyAsync(site_coords, d_coords, 4 * coord_elems, back, s));
-      if (site_top) LG_CUDA(cudaMemcpyAsync(site_top, d_top, 4 * (size_t)L * K, back, s));
-      if (d_out64) LG_CUDA(cudaMemcpyAsync(site_s64, d_out64, 8 * (size_t)L * K, back, s));
+      LG_CUDA(cudaMemcpyAsync(S.site_poses, S.d_poses, 4 * pose_floats, back, s));
+      LG_CUDA(cudaMemcpyAsync(S.site_scores, S.d_scores, 4 * (size_t)L * K, back, s));
+      if (S.d_trace) LG_CUDA(cudaMemcpyAsync(S.site_trace, S.d_trace, 2 * trace_elems, back, s));
+      if (S.d_coords) LG_CUDA(cudaMemcpyAsync(S.site_coords, S.d_coords, 4 * coord_elems, back, s));
+      if (S.site_top) LG_CUDA(cudaMemcpyAsync(S.site_top, S.d_top, 4 * (size_t)L * K, back, s));
+      if (S.d_out64) LG_CUDA(cudaMemcpyAsync(S.site_s64, S.d_out64, 8 * (size_t)L * K, back, s));
     }
     tm.mark();
     tm.finish();
