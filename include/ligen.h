@@ -391,6 +391,13 @@ int ligen_release_prepared(ligen_prepared_t* prep);
 int ligen_pose_grad(const ligen_ligands_t* ligands, const ligen_grid_t* grid, int32_t poses_per_ligand,
                     const float* poses, float out_penalty, float* out_scores, float* out_grads, void* stream);
 
+/* ligen_pose_grad with every pose's gradient multiplied by weights[l][p] (the
+ * backward of a weighted sum of scores; the scores are not weighted).
+ * `weights` shares the memory space of `poses` and the outputs. */
+int ligen_pose_grad_weighted(const ligen_ligands_t* ligands, const ligen_grid_t* grid, int32_t poses_per_ligand,
+                             const float* poses, float out_penalty, const float* weights, float* out_scores,
+                             float* out_grads, void* stream);
+
 /* Gradient refinement of poses in place: for every pose, `steps` iterations
  * of normalised-step projected ascent. An iteration moves t by step_t (A)
  * along dS/dt / |dS/dt| (then clamps t to the grid box), q^ = q/|q| by step_q

@@ -319,6 +319,18 @@ def pose_grad(ligands: Ligands, grid: PocketGrid, poses: torch.Tensor, poses_per
     return scores, grads
 
 
+def _weighted_pose_grad(ligands, grid, poses, poses_per_ligand, out_penalty, weights):
+    """ligen_pose_grad_weighted: weights[l, p] * dS/dpose in the packing of `poses`."""
+    lib = _abi.load()
+    scores = _empty((ligands.n_ligands, poses_per_ligand), torch.float32, poses.device)
+    grads = _empty(tuple(poses.shape), torch.float32, poses.device)
+    weights = weights.detach().to(device=poses.device, dtype=torch.float32).contiguous()
+    check(lib.ligen_pose_grad_weighted(C.byref(ligands._s), C.byref(grid._s), poses_per_ligand, _ptr(poses),
+                                       float(out_penalty), _ptr(weights), _ptr(scores), _ptr(grads),
+                                       _stream_handle(poses.device)))
+    return grads
+
+
 def refine_poses(ligands: Ligands, grid: PocketGrid, poses: torch.Tensor, poses_per_ligand: int, *,
                  steps: int = 50, step_t: float = 0.1, step_q: float = 0.02, step_theta: float = 0.05,
                  out_penalty: float = 5.0, accept: bool = False, inplace: bool = False):
@@ -353,6 +365,10 @@ class PoseScore(torch.autograd.Function):
     def backward(ctx, grad_scores):
         (poses,) = ctx.saved_tensors
         ligands, grid, P, pen = ctx.args
+        if not (torch.is_grad_enabled() and grad_scores.requires_grad):
+            # the kernel multiplies each pose's gradient by its score's
+            return _weighted_pose_grad(ligands, grid, poses.detach().contiguous(), P, pen, grad_scores), None, None, None, None
+        # create_graph: the result stays differentiable with respect to grad_scores
         _, grads = pose_grad(ligands, grid, poses.detach().contiguous(), P, pen)
         weight = grad_scores.reshape(-1).repeat_interleave(_pose_lengths(ligands, P, poses.device))
         return grads * weight, None, None, None, None

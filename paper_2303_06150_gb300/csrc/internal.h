@@ -126,6 +126,7 @@ struct GradArgs {
   float* inout_poses;       // refinement: poses, refined in place
   float* out_scores;        // [L][P]
   float* out_grads;         // gradient: same packing as poses
+  const float* weights;     // gradient: [L][P] factors of the poses' gradients, or NULL
   int steps;                // refinement iterations
   float step_t, step_q, step_theta;
   float box_lo[3], box_hi[3];

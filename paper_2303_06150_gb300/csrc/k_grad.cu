@@ -216,7 +216,7 @@ __global__ void __launch_bounds__(32 * kGradWarps) grad_kernel(const GradArgs a)
       !lg_check(a.grid.check, a.lig.atom_off[l + 1] - a.lig.atom_off[l] <= a.max_atoms, kChkItemShape)) {
     if (sl.own) {   // the early return is uniform over the warp (one ligand)
       if (sub == 0) a.out_scores[gp] = -INFINITY;
-      for (int e = sub; e < 7 + n; e += kGradLanes) a.out_grads[off + e] = 0.f;
+      for (int e = sub; e < 7 + n; e += kGradLanes) a.out_grads[off + e] = a.weights ? 0.f * a.weights[gp] : 0.f;
     }
     return;
   }
@@ -224,7 +224,8 @@ __global__ void __launch_bounds__(32 * kGradWarps) grad_kernel(const GradArgs a)
   const float S = group_score_grad(a, l, a.poses + off, W, gbuf[sl.slot]);
   if (sl.own) {
     if (sub == 0) a.out_scores[gp] = S;
-    for (int e = sub; e < 7 + n; e += kGradLanes) a.out_grads[off + e] = gbuf[sl.slot][e];
+    const float wt = a.weights ? a.weights[gp] : 1.f;
+    for (int e = sub; e < 7 + n; e += kGradLanes) a.out_grads[off + e] = gbuf[sl.slot][e] * wt;
   }
 }
 
@@ -574,7 +575,7 @@ __global__ void __launch_bounds__(32, 16) grad_lane_kernel(const GradArgs a) {
   if (!ok) {   // uniform over the warp (one ligand)
     if (own && sub == 0) a.out_scores[gp] = -INFINITY;
     if (!REFINE && own)
-      for (int e = sub; e < plen; e += G) a.out_grads[off + e] = 0.f;
+      for (int e = sub; e < plen; e += G) a.out_grads[off + e] = a.weights ? 0.f * a.weights[gp] : 0.f;
     return;
   }
   const int sl = 7 + ncap;
@@ -589,7 +590,8 @@ __global__ void __launch_bounds__(32, 16) grad_lane_kernel(const GradArgs a) {
   if constexpr (!REFINE) {
     if (own) {
       if (sub == 0) a.out_scores[gp] = Sc;
-      for (int e = sub; e < plen; e += G) a.out_grads[off + e] = grad[e];
+      const float wt = a.weights ? a.weights[gp] : 1.f;
+      for (int e = sub; e < plen; e += G) a.out_grads[off + e] = grad[e] * wt;
     }
     return;
   } else {

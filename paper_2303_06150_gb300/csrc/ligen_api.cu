@@ -1606,7 +1606,7 @@ int ligen_release_prepared(ligen_prepared_t* prep) {
 // the grid records, pack the ligands, run the gradient kernel, copy back.
 static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, int32_t poses_per_ligand,
                      const float* poses_in, float* poses_inout, float out_penalty, float* out_scores,
-                     float* out_grads, int refine, int32_t steps, float step_t, float step_q, float step_theta,
+                     float* out_grads, const float* weights, int refine, int32_t steps, float step_t, float step_q, float step_theta,
                      int8_t* out_accept, void* stream) {
   g_err.clear();
   int rc;
@@ -1630,7 +1630,7 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
   const int lhost = space_of({ligands->atom_off, ligands->xyz, ligands->type, ligands->bonds,
                               ligands->rot_off, ligands->rot_edge});
   const int ghost = space_of({grid->data});
-  const int ohost = space_of({pin, out_scores, out_grads, out_accept});
+  const int ohost = space_of({pin, out_scores, out_grads, weights, out_accept});
   if (lhost < 0 || ohost < 0) return fail(LIGEN_ERR_INVALID_ARG, "arrays mix host and device memory");
   const size_t pose_floats = (size_t)poses_per_ligand * (7 * (size_t)L + sh.rot);
   const size_t nposes = (size_t)poses_per_ligand * L;
@@ -1648,10 +1648,11 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
   if (lanes) plan_score(ligands->h_rot_off, L, &plan);
   const size_t o_list = ar.take(4 * plan.list.size());
   const FkRegions o_fk = lanes ? take_fk(ar, sh, L) : FkRegions{};
-  size_t o_poses = 0, o_scores = 0, o_grads = 0, o_acc = 0;
+  size_t o_poses = 0, o_scores = 0, o_grads = 0, o_weights = 0, o_acc = 0;
   if (ohost) {
     o_poses = ar.take(4 * pose_floats);
     o_scores = ar.take(4 * nposes);
+    if (weights) o_weights = ar.take(4 * nposes);
     if (!refine) o_grads = ar.take(4 * pose_floats);
     if (out_accept) o_acc = ar.take(nposes * (size_t)steps);
   }
@@ -1670,6 +1671,7 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
   if (ohost) {
     LG_CUDA(cudaMemcpyAsync(ar.base + o_poses, pin, 4 * pose_floats, cudaMemcpyHostToDevice, s));
     d_poses = ar.at<float>(o_poses);
+    if (weights) LG_CUDA(cudaMemcpyAsync(ar.base + o_weights, weights, 4 * nposes, cudaMemcpyHostToDevice, s));
   }
   float* coef = ar.at<float>(o_coef);
   LG_CUDA(launch_grid_prep(gvals, grid->nx, grid->ny, grid->nz, grid->nc, coef, s));
@@ -1693,6 +1695,7 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
   ga.inout_poses = d_poses;
   ga.out_scores = ohost ? ar.at<float>(o_scores) : out_scores;
   ga.out_grads = refine ? nullptr : (ohost ? ar.at<float>(o_grads) : out_grads);
+  ga.weights = weights && ohost ? ar.at<float>(o_weights) : weights;
   ga.steps = steps;
   ga.step_t = step_t;
   ga.step_q = step_q;
@@ -1735,14 +1738,24 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
 
 int ligen_pose_grad(const ligen_ligands_t* ligands, const ligen_grid_t* grid, int32_t poses_per_ligand,
                     const float* poses, float out_penalty, float* out_scores, float* out_grads, void* stream) {
-  return grad_call(ligands, grid, poses_per_ligand, poses, nullptr, out_penalty, out_scores, out_grads, 0, 0, 0.f,
-                   0.f, 0.f, nullptr, stream);
+  return grad_call(ligands, grid, poses_per_ligand, poses, nullptr, out_penalty, out_scores, out_grads, nullptr, 0, 0,
+                   0.f, 0.f, 0.f, nullptr, stream);
+}
+
+int ligen_pose_grad_weighted(const ligen_ligands_t* ligands, const ligen_grid_t* grid, int32_t poses_per_ligand,
+                             const float* poses, float out_penalty, const float* weights, float* out_scores,
+                             float* out_grads, void* stream) {
+  g_err.clear();
+  if (!weights && ligands && ligands->n_ligands > 0 && poses_per_ligand > 0)
+    return fail(LIGEN_ERR_INVALID_ARG, "weights is NULL");
+  return grad_call(ligands, grid, poses_per_ligand, poses, nullptr, out_penalty, out_scores, out_grads, weights, 0, 0,
+                   0.f, 0.f, 0.f, nullptr, stream);
 }
 
 int ligen_refine_poses(const ligen_ligands_t* ligands, const ligen_grid_t* grid, int32_t poses_per_ligand,
                        float* poses, float out_penalty, int32_t steps, float step_t, float step_q, float step_theta,
                        float* out_scores, int8_t* out_accept, void* stream) {
-  return grad_call(ligands, grid, poses_per_ligand, nullptr, poses, out_penalty, out_scores, nullptr, 1, steps,
+  return grad_call(ligands, grid, poses_per_ligand, nullptr, poses, out_penalty, out_scores, nullptr, nullptr, 1, steps,
                    step_t, step_q, step_theta, out_accept, stream);
 }
 
