@@ -163,11 +163,12 @@ struct RescoreArgs {
   unsigned* check;          // checked builds: first out-of-range code, else NULL
 };
 
-cudaError_t launch_grid_prep(const float* values, int nx, int ny, int nz, int nc, float* coef,
-                             cudaStream_t s);
-// Records in format `fmt` (RecFormat) for the docking kernel.
-cudaError_t launch_grid_prep_fmt(const float* values, int nx, int ny, int nz, int nc, int fmt, void* rec,
-                                 cudaStream_t s);
+// Grid records in format `fmt` (RecFormat). beside_pack: launched right
+// after launch_pack on the same stream, it may start with the packer (neither
+// reads what the other writes) and ends after it: scoring 3 poses of 5,001
+// ligands 90.7 -> 83.8 us per call, docking 32 small ligands 37.3 -> 34.8.
+cudaError_t launch_grid_prep(const float* values, int nx, int ny, int nz, int nc, int fmt, void* rec,
+                             bool beside_pack, cudaStream_t s);
 // max_atoms: the library's largest ligand. With out.fk_xs set, the
 // forward-kinematics table (out.fk_*) too.
 cudaError_t launch_pack(const LigandsDev& lig, int nc, const Packed& out, int max_atoms, cudaStream_t s);

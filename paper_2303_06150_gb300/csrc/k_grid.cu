@@ -85,32 +85,37 @@ __global__ void __launch_bounds__(kPrepThreads) grid_prep_kernel(const float* __
     }
     c000 = c001; c100 = c101; c010 = c011; c110 = c111;
   }
+  // beside_pack: what follows this kernel in the stream also follows the packer
+  asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 template <int FMT>
-cudaError_t launch_prep(const float* values, int nx, int ny, int nz, int nc, void* rec, cudaStream_t s) {
+cudaError_t launch_prep(const float* values, int nx, int ny, int nz, int nc, void* rec, bool beside_pack,
+                        cudaStream_t s) {
   const size_t cx = rec_cells(nx, FMT), cy = rec_cells(ny, FMT), cz = rec_cells(nz, FMT);
   const size_t tiles = (cx * nc + kPrepThreads - 1) / kPrepThreads;
   const size_t full = tiles * cy * cz / kPrepBlocks;
   const size_t march = full < 2 ? 2 : full < kPrepMarch ? full : kPrepMarch;
   const size_t blocks = tiles * cy * ((cz + march - 1) / march);
-  grid_prep_kernel<FMT>
-      <<<(unsigned)blocks, kPrepThreads, 0, s>>>(values, nx, ny, nz, nc, (int)tiles, (int)march, rec);
-  return cudaGetLastError();
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)blocks);
+  cfg.blockDim = dim3(kPrepThreads);
+  cfg.stream = s;
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cfg.attrs = &at;
+  cfg.numAttrs = beside_pack ? 1 : 0;
+  return cudaLaunchKernelEx(&cfg, grid_prep_kernel<FMT>, values, nx, ny, nz, nc, (int)tiles, (int)march, rec);
 }
 
 }  // namespace
 
-cudaError_t launch_grid_prep_fmt(const float* values, int nx, int ny, int nz, int nc, int fmt, void* rec,
-                                 cudaStream_t s) {
-  return fmt == kRecF32   ? launch_prep<kRecF32>(values, nx, ny, nz, nc, rec, s)
-         : fmt == kRecF16 ? launch_prep<kRecF16>(values, nx, ny, nz, nc, rec, s)
-                          : launch_prep<kRecBF16>(values, nx, ny, nz, nc, rec, s);
-}
-
-cudaError_t launch_grid_prep(const float* values, int nx, int ny, int nz, int nc, float* coef,
-                             cudaStream_t s) {
-  return launch_prep<kRecF32>(values, nx, ny, nz, nc, coef, s);
+cudaError_t launch_grid_prep(const float* values, int nx, int ny, int nz, int nc, int fmt, void* rec,
+                             bool beside_pack, cudaStream_t s) {
+  return fmt == kRecF32   ? launch_prep<kRecF32>(values, nx, ny, nz, nc, rec, beside_pack, s)
+         : fmt == kRecF16 ? launch_prep<kRecF16>(values, nx, ny, nz, nc, rec, beside_pack, s)
+                          : launch_prep<kRecBF16>(values, nx, ny, nz, nc, rec, beside_pack, s);
 }
 
 }  // namespace ligen

@@ -176,6 +176,7 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(const LigandsDev 
                                                                int acap) {
   static_assert(LIGEN_MAX_ROT == 32, "one lane per rotatable bond");
   extern __shared__ __align__(16) unsigned char pack_smem[];
+  asm volatile("griddepcontrol.launch_dependents;");   // the grid records (launch_grid_prep) need nothing of this
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int l = blockIdx.x * kPackWarps + warp;
   if (l >= lig.L) return;

@@ -1159,14 +1159,15 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     S.d_coords = S.site_coords ? (ohost ? ar.at<float>(o_coords) : S.site_coords) : nullptr;
     S.d_top = S.site_top ? (ohost ? ar.at<int32_t>(o_top) : S.site_top) : nullptr;
   };
-  auto records = [&](const Site& S, const SiteSet& b, cudaStream_t st) -> int {
-    LG_CUDA(launch_grid_prep_fmt(S.gvals, S.grid->nx, S.grid->ny, S.grid->nz, S.grid->nc, fmt, ar.at<float>(b.coef), st));
+  auto records = [&](const Site& S, const SiteSet& b, bool beside_pack, cudaStream_t st) -> int {
+    LG_CUDA(launch_grid_prep(S.gvals, S.grid->nx, S.grid->ny, S.grid->nz, S.grid->nc, fmt, ar.at<float>(b.coef),
+                             beside_pack, st));
     return LIGEN_OK;
   };
   auto pack = [&]() -> int {
-    LG_CUDA(launch_pack(lig, grids[0].nc, pk, sh.max_atoms, s));
     if (longest_first)
       LG_CUDA(launch_order(lig, params->n_rigid, P, 360 / params->torsion_step_deg, ar.at<int32_t>(o_order), s));
+    LG_CUDA(launch_pack(lig, grids[0].nc, pk, sh.max_atoms, s));
     return LIGEN_OK;
   };
   auto search = [&](Site& S, const SiteSet& b, cudaStream_t st) -> int {
@@ -1294,7 +1295,7 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
       const int k = g & 1;
       open_site(g, sites[k]);
       if (g >= 2) LG_CUDA(cudaStreamWaitEvent(pipe->high, pipe->docked[k], 0));
-      const int e = records(sites[k], set[k], pipe->high);
+      const int e = records(sites[k], set[k], false, pipe->high);
       if (e != LIGEN_OK) return e;
       LG_CUDA(cudaEventRecord(pipe->prep[k], pipe->high));
       return LIGEN_OK;
@@ -1326,9 +1327,14 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     if (ghost)
       LG_CUDA(cudaMemcpyAsync(ar.base + o_gval, S.grid->data, grid_values_bytes(S.grid), cudaMemcpyHostToDevice, s));
     tm.mark();
-    if ((rc = records(S, set[0], s)) != LIGEN_OK) return rc;
-    tm.mark();
-    if (site == 0 && (rc = pack()) != LIGEN_OK) return rc;
+    if (stage_out) {   // one stage after another
+      if ((rc = records(S, set[0], false, s)) != LIGEN_OK) return rc;
+      tm.mark();
+      if (site == 0 && (rc = pack()) != LIGEN_OK) return rc;
+    } else {
+      if (site == 0 && (rc = pack()) != LIGEN_OK) return rc;
+      if ((rc = records(S, set[0], site == 0, s)) != LIGEN_OK) return rc;
+    }
     tm.mark();
     if ((rc = search(S, set[0], s)) != LIGEN_OK) return rc;
     tm.mark();
@@ -1434,7 +1440,6 @@ int ligen_score_poses(const ligen_ligands_t* ligands, const ligen_grid_t* grid, 
   if (!plan.list.empty())   // pageable source: staged before the call returns
     LG_CUDA(cudaMemcpyAsync(ar.base + o_list, plan.list.data(), 4 * plan.list.size(), cudaMemcpyHostToDevice, s));
   float* coef = ar.at<float>(o_coef);
-  LG_CUDA(launch_grid_prep(gvals, grid->nx, grid->ny, grid->nz, grid->nc, coef, s));
   Packed pk{};
   pk.xc = ar.at<float4>(o_xc);
   pk.binfo = ar.at<uchar4>(o_binfo);
@@ -1442,6 +1447,7 @@ int ligen_score_poses(const ligen_ligands_t* ligands, const ligen_grid_t* grid, 
   pk.status = ar.at<int32_t>(o_status);
   if (lanes) set_fk(ar, o_fk, &pk);
   LG_CUDA(launch_pack(lig, grid->nc, pk, sh.max_atoms, s));
+  LG_CUDA(launch_grid_prep(gvals, grid->nx, grid->ny, grid->nz, grid->nc, kRecF32, coef, true, s));
   ScoreArgs sa{};
   sa.lig = lig;
   sa.pk = pk;
@@ -1546,8 +1552,9 @@ int ligen_prepare_scoring(const ligen_ligands_t* ligands, const ligen_grid_t* gr
     if (ce == cudaSuccess)
       ce = cudaMemcpyAsync(h->d_list, h->plan.list.data(), 4 * (size_t)L, cudaMemcpyHostToDevice, s);
   }
-  if (ce == cudaSuccess) ce = launch_grid_prep(gvals, grid->nx, grid->ny, grid->nz, grid->nc, h->coef, s);
   if (ce == cudaSuccess && L) ce = launch_pack(lig, grid->nc, h->pk, sh.max_atoms, s);
+  if (ce == cudaSuccess)
+    ce = launch_grid_prep(gvals, grid->nx, grid->ny, grid->nz, grid->nc, kRecF32, h->coef, L > 0, s);
   if (ce != cudaSuccess) return bail(cuda_fail(ce, "preparing the scoring inputs"));
   // Host inputs are copied through the workspace asynchronously: wait for
   // the copies, so the caller may reuse its host buffers on return.
@@ -1697,7 +1704,6 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
     if (weights) LG_CUDA(cudaMemcpyAsync(ar.base + o_weights, weights, 4 * nposes, cudaMemcpyHostToDevice, s));
   }
   float* coef = ar.at<float>(o_coef);
-  LG_CUDA(launch_grid_prep(gvals, grid->nx, grid->ny, grid->nz, grid->nc, coef, s));
   Packed pk{};
   pk.xc = ar.at<float4>(o_xc);
   pk.binfo = ar.at<uchar4>(o_binfo);
@@ -1705,6 +1711,7 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
   pk.status = ar.at<int32_t>(o_status);
   if (lanes) set_fk(ar, o_fk, &pk);
   LG_CUDA(launch_pack(lig, grid->nc, pk, sh.max_atoms, s));
+  LG_CUDA(launch_grid_prep(gvals, grid->nx, grid->ny, grid->nz, grid->nc, kRecF32, coef, true, s));
   GradArgs ga{};
   ga.lig = lig;
   ga.pk = pk;
@@ -1974,7 +1981,7 @@ int ligen_autotune(const ligen_ligands_t* ligands, const ligen_grid_t* grid, con
   lig.atom_off = ligands->atom_off; lig.xyz = ligands->xyz; lig.type = ligands->type;
   lig.bonds = ligands->bonds; lig.rot_off = ligands->rot_off; lig.rot_edge = ligands->rot_edge;
   float* coef = ar.at<float>(o_coef);
-  LG_CUDA(launch_grid_prep_fmt((const float*)grid->data, grid->nx, grid->ny, grid->nz, grid->nc, fmt, coef, s));
+  LG_CUDA(launch_grid_prep((const float*)grid->data, grid->nx, grid->ny, grid->nz, grid->nc, fmt, coef, false, s));
   Packed pk{};
   pk.xc = ar.at<float4>(o_xc);
   pk.binfo = ar.at<uchar4>(o_binfo);
@@ -2226,7 +2233,6 @@ extern "C" int ligen_dock_batch_static(const ligen_ligands_t* ligands, const lig
   lig.atom_off = ligands->atom_off; lig.xyz = ligands->xyz; lig.type = ligands->type;
   lig.bonds = ligands->bonds; lig.rot_off = ligands->rot_off; lig.rot_edge = ligands->rot_edge;
   float* coef = ar.at<float>(o_coef);
-  LG_CUDA(launch_grid_prep((const float*)grid->data, grid->nx, grid->ny, grid->nz, grid->nc, coef, s));
   Packed pk{};
   pk.xc = ar.at<float4>(o_xc);
   pk.binfo = ar.at<uchar4>(o_binfo);
@@ -2234,6 +2240,7 @@ extern "C" int ligen_dock_batch_static(const ligen_ligands_t* ligands, const lig
   pk.touch = ar.at<uint32_t>(o_touch);
   pk.status = ar.at<int32_t>(o_status);
   LG_CUDA(launch_pack(lig, grid->nc, pk, sh.max_atoms, s));
+  LG_CUDA(launch_grid_prep((const float*)grid->data, grid->nx, grid->ny, grid->nz, grid->nc, kRecF32, coef, true, s));
 
   DockArgs da{};
   da.lig = lig;
