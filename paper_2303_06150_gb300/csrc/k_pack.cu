@@ -262,31 +262,42 @@ __global__ void __launch_bounds__(32 * kPackWarps) pack_kernel(const LigandsDev 
   __syncwarp();
 
   if (!bad) {
-    // the walk from atom 0; an edge is used when exactly one end was seen
+    // The walk from atom 0; an edge is used when exactly one end was seen.
+    // Edges and their bonds are in registers and a round's reads
+    // unconditional, so a round is two shared-memory latencies whatever W
+    // (with the reads behind each edge's own test a round was eight).
     if (lane < n) atomicOr(&S.emask[myedge], 1u << lane);
+    __syncwarp();
+    unsigned edge[W], bonds[W];
     unsigned left = 0u;   // this lane's unused edges, bit w
 #pragma unroll
-    for (int w = 0; w < W; ++w)
-      if (32 * w + lane < N - 1) left |= 1u << w;
-    __syncwarp();
+    for (int w = 0; w < W; ++w) {
+      edge[w] = bonds[w] = 0u;   // no edge: atom 0 to itself, never used
+      if (32 * w + lane < N - 1) {
+        edge[w] = S.edge[32 * w + lane];
+        bonds[w] = S.emask[32 * w + lane];
+        left |= 1u << w;
+      }
+    }
     while (true) {   // every round with progress uses an edge: at most N - 1 rounds
       unsigned use = 0u, child_b = 0u;
 #pragma unroll
-      for (int w = 0; w < W; ++w)
-        if (left >> w & 1u) {
-          const unsigned e = S.edge[32 * w + lane];
-          const bool sa = S.seen[e & 0xffu], sb = S.seen[e >> 8];
-          if (sa != sb) use |= 1u << w;
-          if (sa) child_b |= 1u << w;
-        }
+      for (int w = 0; w < W; ++w) {
+        const unsigned sa = S.seen[edge[w] & 0xffu], sb = S.seen[edge[w] >> 8];
+        use |= (sa ^ sb) << w;
+        child_b |= sa << w;
+      }
+      use &= left;
       if (!__any_sync(kFull, use != 0u)) break;
+      unsigned path[W];
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        path[w] = S.path[child_b >> w & 1u ? edge[w] & 0xffu : edge[w] >> 8] | bonds[w];
 #pragma unroll
       for (int w = 0; w < W; ++w)
         if (use >> w & 1u) {
-          const unsigned e = S.edge[32 * w + lane];
-          const unsigned ch = child_b >> w & 1u ? e >> 8 : e & 0xffu;
-          const unsigned pa = child_b >> w & 1u ? e & 0xffu : e >> 8;
-          S.path[ch] = S.path[pa] | S.emask[32 * w + lane];
+          const unsigned ch = child_b >> w & 1u ? edge[w] >> 8 : edge[w] & 0xffu;
+          S.path[ch] = path[w];
           S.seen[ch] = 1;
         }
       left &= ~use;
