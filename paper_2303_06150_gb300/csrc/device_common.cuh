@@ -275,35 +275,6 @@ __device__ __forceinline__ float grid_sample(const GridView& g, float ux, float 
   return e;
 }
 
-// grid_sample without a branch around the load: the position is clamped
-// into the box first, so the record address is always valid and the load
-// is unconditional (the compiler can issue the loads of several atoms
-// before using any), and the penalty is selected afterwards for a point
-// outside the box. Inside the box the clamp changes nothing and the value
-// is grid_sample's, bit for bit; a NaN coordinate clamps to 0 and takes the
-// penalty, as in grid_sample.
-__device__ __forceinline__ float grid_sample_nb(const GridView& g, float ux, float uy, float uz, int c) {
-  const bool inb = (ux >= 0.f) & (ux <= g.mx) & (uy >= 0.f) & (uy <= g.my) & (uz >= 0.f) & (uz <= g.mz);
-  const float vx = fminf(fmaxf(ux, 0.f), g.mx), vy = fminf(fmaxf(uy, 0.f), g.my), vz = fminf(fmaxf(uz, 0.f), g.mz);
-  const float fx = fminf(floorf(vx), g.mx - 1.f);
-  const float fy = fminf(floorf(vy), g.my - 1.f);
-  const float fz = fminf(floorf(vz), g.mz - 1.f);
-  const int ix = (int)fx, iy = (int)fy, iz = (int)fz;
-  const float dx = vx - fx, dy = vy - fy, dz = vz - fz;
-  const size_t ri = rec_index(g.cx, g.cy, g.cz, c, ix, iy, iz);
-  if (!lg_check(g.check, c >= 0 && c < g.nc && ri < g.n_rec, kChkGridRecord)) return g.penalty;
-  float a[8];
-  ld_global_v8_na(g.coef + ri * 8, a);
-  const float t1 = fmaf(dz, a[7], a[4]);
-  float t2 = fmaf(dy, t1, a[1]);
-  t2 = fmaf(dz, a[5], t2);
-  const float t3 = fmaf(dz, a[6], a[2]);
-  float e = fmaf(dz, a[3], a[0]);
-  e = fmaf(dy, t3, e);
-  e = fmaf(dx, t2, e);
-  return inb ? e : g.penalty;
-}
-
 // Grid record formats of the docking kernel.
 //   kRecF32:  32-byte records, the 8 FP32 coefficients of the cell's
 //             trilinear polynomial (one 256-bit load, 7 FMA);
@@ -401,9 +372,9 @@ __device__ __forceinline__ float grid_sample_fmt(const GridView& g, float ux, fl
 //
 // Measured on GB300 against floorf, conversions, six comparisons and a clamp
 // per scalar sample (docking kernel, 12,000 screening / 3,000 bimodal
-// ligands): FP32 26.28 -> 23.00 / 11.93 -> 9.59 ms (2,000 screening ligands:
+// ligands): FP32 26.28 -> 23.12 / 11.93 -> 9.66 ms (2,000 screening ligands:
 // 3.67 -> 2.44 G warp instructions, 4.69 -> 3.88 ms, 303 G samples/s of the
-// 308 G/s gather ceiling), FP16 26.25 -> 25.26 / 11.76 -> 11.22 ms.
+// 308 G/s gather ceiling), FP16 26.25 -> 25.28 / 11.76 -> 11.23 ms.
 constexpr float kFloorMagic = 8388608.f;   // 2^23
 
 struct DockPoint {   // a position, its cell as unreduced bits, its fractions

@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(32 * kScoreWarps, 8) score_kernel(const ScoreA
 // builds the n + 1 transforms of its pose, 48 bytes each, in shared memory
 // [slot][pose][12] (a 48-byte stride keeps 128-bit accesses free of bank
 // conflicts); per atom one 3x4 transform of its owner (9 FMA) and one
-// branch-free record load, 8 in flight per lane. Shared memory grows with
+// branch-free record load, 4 in flight per lane. Shared memory grows with
 // the bonds, so the caller launches ligands by rotatable-bond class. Groups
 // past the ligand's last pose shadow it and write nothing.
 template <int G>
@@ -153,14 +153,17 @@ __device__ __forceinline__ void score_lane_item(const ScoreArgs& a, size_t gw, c
     fk_transforms(S, n, pt, q, Tg, stride, a.origin, a.inv_h, Tg, stride);
   }
   if (G > 1) __syncwarp();
-  // samples: unconditional loads, 8 gathers in flight per lane. The atoms
+  // samples: unconditional loads, 4 gathers in flight per lane (88 registers;
+  // the 600,000-pose call 131 us, 133 with 8 in flight by the sampler before
+  // grid_fetch, 150 with 8 now; padded batches of 4, 6 and 8 instead of a
+  // remainder loop 139, 141 and 158). The atoms
   // are listed by owner, so the owner's transform stays in registers across
   // its atoms and is read again only where the owner changes (a uniform
   // branch: every lane is at the same atom).
   float acc = 0.f;
   int cur = -1;
   float4 m0, m1, m2;
-#pragma unroll 8
+#pragma unroll 4
   for (int i = sub; i < N; i += G) {
     const float4 X = S.sx[i];
     const int o = S.own[i];
@@ -171,7 +174,7 @@ __device__ __forceinline__ void score_lane_item(const ScoreArgs& a, size_t gw, c
     const float ux = fmaf(m0.x, X.x, fmaf(m0.y, X.y, fmaf(m0.z, X.z, m0.w)));
     const float uy = fmaf(m1.x, X.x, fmaf(m1.y, X.y, fmaf(m1.z, X.z, m1.w)));
     const float uz = fmaf(m2.x, X.x, fmaf(m2.y, X.y, fmaf(m2.z, X.z, m2.w)));
-    acc -= grid_sample_nb(a.grid, ux, uy, uz, __float_as_int(X.w));
+    acc -= fetched_value(a.grid, grid_fetch(a.grid, ux, uy, uz, __float_as_int(X.w)));
   }
 #pragma unroll
   for (int o = G / 2; o > 0; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
@@ -182,7 +185,7 @@ __device__ __forceinline__ void score_lane_item(const ScoreArgs& a, size_t gw, c
 // blockIdx.x, blockIdx.x + gridDim.x, ... (one CTA per item left the
 // block scheduler starting 20,000 one-warp CTAs per call).
 template <int G>
-__global__ void __launch_bounds__(32, 16) score_lane_kernel(const ScoreArgs a) {
+__global__ void __launch_bounds__(32, 20) score_lane_kernel(const ScoreArgs a) {
   extern __shared__ __align__(16) unsigned char lane_smem[];
   FkLigand S;
   float* T;
