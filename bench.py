@@ -555,11 +555,12 @@ def run_ours(args):
               "roofline": roofline,
               "gpu_launches": None,
               "clocks": best["clocks"]}
-    # our kernels per step: grid preparation, packer, top-K, and one docking
-    # launch (plain) or one per (atom class, kernel shape) group (buckets)
+    # our kernels per step: grid preparation, packer, top-K, and the ligand
+    # order and one docking launch (plain) or one per (atom class, kernel
+    # shape) group (buckets); the re-score adds its table, itself and the re-rank
     table = lg.tune_get()
-    per_step = (3 + (len({(b // 11, table[b]) for b in present}) if FORMS[form]["batching"] != "plain" else 1)
-                + int(bool(FORMS[form].get("rescore_fp64"))))
+    per_step = (3 + (len({(b // 11, table[b]) for b in present}) if FORMS[form]["batching"] != "plain" else 2)
+                + 3 * int(bool(FORMS[form].get("rescore_fp64"))))
     result["gpu_launches"] = per_step * args.steps
     if tuned is not None:
         result["tuning"] = {str(b): list(v[:2]) for b, v in sorted(tuned.items())}
@@ -609,10 +610,10 @@ def run_ours(args):
             "relative_gain_mean": float(np.mean(gain / np.maximum(np.abs(b), 1e-6))),
             "improved_fraction": float((gain > 0).mean()),
             "best_pose_gain_mean": float((after.max(1).values - before.max(1).values).mean().item()),
-            "launches_per_call": 3 + score_classes(lib),
+            "launches_per_call": 2 + score_classes(lib),
             "how": "top-16 poses per ligand of the sweep, normalised-step projected ascent "
-                   "(0.1 A, 0.02, 0.05 rad; halve on rejection); per call grid preparation, packer, "
-                   "forward-kinematics table and one refinement launch per rotatable-bond class "
+                   "(0.1 A, 0.02, 0.05 rad; halve on rejection); per call grid preparation, packer "
+                   "(with the forward-kinematics table) and one refinement launch per rotatable-bond class "
                    "(side by side on forked streams), timed with CUDA events (best of 3)"}
 
     if args.workload == "screen20k":
@@ -651,8 +652,8 @@ def run_ours(args):
             "gather_peak_loads_per_s": probe32["loads_per_s"],
             "launches_per_call": score_classes(lib),
             "how": "ligen_score_poses on the kept poses of the timed form (20,000 ligands x top 30), FP32 grid "
-                   "records: 'ms' is the whole call (grid records, packer, forward-kinematics table, scoring "
-                   "launches), 'kernel_ms' the whole ligen_score_prepared call on inputs prepared once (one "
+                   "records: 'ms' is the whole call (grid records, packer with the forward-kinematics table, "
+                   "scoring launches), 'kernel_ms' the whole ligen_score_prepared call on inputs prepared once (one "
                    "launch per rotatable-bond class, side by side, replayed from a CUDA graph; host issue "
                    "included); CUDA events, best of 3 and 10; frac_gather = atom samples/s over the 32-byte "
                    "random-gather probe's loads/s, frac_l2 = 32 bytes per sample over the streaming L2 "

@@ -588,9 +588,9 @@ const Shape kBigShapes[] = {LG_BIG(kRecF32), LG_BIG(kRecF16), LG_BIG(kRecBF16)};
 // Shared memory the resident CTAs may take together (of the SM's 256 KB of
 // L1 and shared memory), and the build for a CTA of `smem` bytes: the one
 // asking for as many CTAs as fit that budget. 192 KB puts the screening
-// library (~20 KB per CTA) at 8 CTAs and the bimodal one (27.6 KB, with the
-// host's upper bound on the moving lists) at 7, the best of the measured
-// builds for each.
+// library (~20 KB per CTA) at the 8-CTA build (7 CTAs for five-slot FP32
+// shapes) and the bimodal one (27.6 KB, with the host's upper bound on the
+// moving lists) at 7, the best of the measured builds for each.
 constexpr size_t kCtaSmemBudget = 192 * 1024;
 int build_for(size_t smem) {
   const size_t fit = smem ? kCtaSmemBudget / smem : 8;

@@ -8,7 +8,7 @@
 // the cell below and every step costs four loads (consecutive threads:
 // consecutive channels, then x; whole lines), twelve additions and one store
 // of the whole record; indices are divided out once per thread. Measured on
-// GB300, 96^3 x 8: FP32 63 -> 42 us (5.9 TB/s), FP16 66 -> 27 us, against
+// GB300, 96^3 x 8: FP32 63 -> 40.5 us (6.1 TB/s), FP16 66 -> 35 us, against
 // one thread per record with 64-bit divisions and eight loads each.
 #include "internal.h"
 

@@ -18,10 +18,11 @@
 // sides, lists and touch masks are popcounts and shuffles. N - 1 edges that
 // reach every atom are a tree, so the walk is the validity check too.
 // Measured on GB300 against one lane walking the tree depth first with
-// per-atom loops, and the table in a kernel of its own: ligen_pack_ligands
-// on 50,000 bimodal ligands (45 atoms, 8 bonds on average) 490 -> 167 us per
-// call, scoring 3 poses of 5,001 screening ligands 142 -> 112 us, docking 32
-// small ligands 77.7 -> 71.5 us.
+// per-atom loops, and the table in a kernel of its own (kernel time): 20,000
+// screening ligands 133 -> 45 us, with the table 126 + 57 -> 54 us; five
+// ligands 33 -> 13 us. ligen_pack_ligands on 50,000 bimodal ligands (45
+// atoms, 8 bonds on average) 490 -> 84 us per call, the host's size checks
+// included.
 #include "../../include/ligen.h"
 #include "internal.h"
 
