@@ -11,6 +11,7 @@ from dataclasses import dataclass
 
 import numpy as np
 import torch
+from torch.autograd import forward_ad
 
 from . import _abi
 from ._abi import GridT, LigandsT, ParamsT, check
@@ -351,6 +352,15 @@ def _pose_lengths(ligands: Ligands, poses_per_ligand: int, device) -> torch.Tens
     return n.repeat_interleave(poses_per_ligand).to(device)
 
 
+def _kernel_reads(t: torch.Tensor) -> bool:
+    """Whether t's memory is all there is to it: no graph to extend, no vmap
+    level, no forward-mode tangent, no subclass, no dispatch mode watching."""
+    return (type(t) is torch.Tensor and not (torch.is_grad_enabled() and t.requires_grad)
+            and torch._C._has_storage(t) and not torch._C._functorch.is_functorch_wrapped_tensor(t)
+            and forward_ad._current_level < 0
+            and torch._C._len_torch_dispatch_stack() == 0)
+
+
 class PoseScore(torch.autograd.Function):
     """Differentiable pose score: forward ligen_score_poses, backward
     ligen_pose_grad (coordinates rebuilt in the backward pass)."""
@@ -365,10 +375,9 @@ class PoseScore(torch.autograd.Function):
     def backward(ctx, grad_scores):
         (poses,) = ctx.saved_tensors
         ligands, grid, P, pen = ctx.args
-        if not (torch.is_grad_enabled() and grad_scores.requires_grad):
-            # the kernel multiplies each pose's gradient by its score's
+        if _kernel_reads(grad_scores):   # the kernel multiplies each pose's gradient by its score's
             return _weighted_pose_grad(ligands, grid, poses.detach().contiguous(), P, pen, grad_scores), None, None, None, None
-        # create_graph: the result stays differentiable with respect to grad_scores
+        # create_graph, vmap (is_grads_batched), forward mode: torch multiplies
         _, grads = pose_grad(ligands, grid, poses.detach().contiguous(), P, pen)
         weight = grad_scores.reshape(-1).repeat_interleave(_pose_lengths(ligands, P, poses.device))
         return grads * weight, None, None, None, None
