@@ -1288,7 +1288,6 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     if (params->status)
       LG_CUDA(cudaMemcpyAsync(params->status, pk.status, 4 * (size_t)L, cudaMemcpyDeviceToDevice, s));
     LG_CUDA(cudaEventRecord(pipe->packed, s));
-    for (cudaStream_t d : pipe->dock) LG_CUDA(cudaStreamWaitEvent(d, pipe->packed, 0));
     std::vector<Site> sites(2);
     // records of site g: when site g - 2 has docked on the same set
     auto prepare = [&](int g) -> int {
@@ -1300,20 +1299,32 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
       LG_CUDA(cudaEventRecord(pipe->prep[k], pipe->high));
       return LIGEN_OK;
     };
-    if ((rc = prepare(0)) != LIGEN_OK) return rc;
-    for (int g = 0; g < n_sites; ++g) {
-      const int k = g & 1;
-      LG_CUDA(cudaStreamWaitEvent(pipe->dock[k], pipe->prep[k], 0));
-      if (g >= 2) LG_CUDA(cudaStreamWaitEvent(pipe->dock[k], pipe->top[k], 0));   // site g - 2's results were read
-      if ((rc = search(sites[k], set[k], pipe->dock[k])) != LIGEN_OK) return rc;
-      LG_CUDA(cudaEventRecord(pipe->docked[k], pipe->dock[k]));
-      if (g + 1 < n_sites && (rc = prepare(g + 1)) != LIGEN_OK) return rc;
-      LG_CUDA(cudaStreamWaitEvent(pipe->high, pipe->docked[k], 0));
-      if ((rc = winners(sites[k], set[k], pipe->high)) != LIGEN_OK) return rc;
-      LG_CUDA(cudaEventRecord(pipe->top[k], pipe->high));
-    }
-    LG_CUDA(cudaEventRecord(pipe->end, pipe->high));   // after every site's docking and winners
-    LG_CUDA(cudaStreamWaitEvent(s, pipe->end, 0));
+    auto run_sites = [&]() -> int {
+      for (cudaStream_t d : pipe->dock) LG_CUDA(cudaStreamWaitEvent(d, pipe->packed, 0));
+      int e = prepare(0);
+      for (int g = 0; g < n_sites && e == LIGEN_OK; ++g) {
+        const int k = g & 1;
+        LG_CUDA(cudaStreamWaitEvent(pipe->dock[k], pipe->prep[k], 0));
+        if (g >= 2) LG_CUDA(cudaStreamWaitEvent(pipe->dock[k], pipe->top[k], 0));   // site g - 2's results were read
+        if ((e = search(sites[k], set[k], pipe->dock[k])) != LIGEN_OK) break;
+        LG_CUDA(cudaEventRecord(pipe->docked[k], pipe->dock[k]));
+        if (g + 1 < n_sites && (e = prepare(g + 1)) != LIGEN_OK) break;
+        LG_CUDA(cudaStreamWaitEvent(pipe->high, pipe->docked[k], 0));
+        if ((e = winners(sites[k], set[k], pipe->high)) != LIGEN_OK) break;
+        LG_CUDA(cudaEventRecord(pipe->top[k], pipe->high));
+      }
+      return e;
+    };
+    rc = run_sites();
+    // The caller's stream goes on after everything that was launched, also
+    // where a launch failed: its next call uses the same workspace.
+    for (int k = 0; k < 2 && rc != LIGEN_OK; ++k)
+      if (cudaEventRecord(pipe->docked[k], pipe->dock[k]) == cudaSuccess)
+        cudaStreamWaitEvent(s, pipe->docked[k], 0);
+    cudaError_t joined = cudaEventRecord(pipe->end, pipe->high);   // after every site's docking and winners
+    if (joined == cudaSuccess) joined = cudaStreamWaitEvent(s, pipe->end, 0);
+    if (rc != LIGEN_OK) return rc;
+    LG_CUDA(joined);
   }
   for (int site = 0; site < n_sites && !overlap; ++site) {
     Site S;
