@@ -180,7 +180,9 @@ size_t dock_smem_bytes(int max_atoms, int max_rot, int max_frag, int rpc);
 int dock_pick_lanes(const int32_t* h_atom_off, const int32_t* h_rot_off, int L, int R, int n_rigid, int n_theta,
                     int passes, int fmt, int sms);
 bool dock_lanes_supported(int lanes);
-// A grid axis of 2^23 cells or more: docked by the 8-lane shapes only.
+// A grid axis of 2^23 cells or more, past the floor by addition of
+// dock_point and grid_fetch: docked by the 8-lane shapes only, poses scored
+// and refined by the group-per-pose kernels.
 inline bool dock_big(const GridView& g) { return g.mx >= kFloorMagic || g.my >= kFloorMagic || g.mz >= kFloorMagic; }
 bool dock_shape_supported(int lanes, int fmt, bool big);
 // grid_ctas: CTAs of a persistent launch (ignored when a.queue is NULL).

@@ -371,6 +371,11 @@ int dock_restarts_per_cta(int R, int lanes) {
   return rpc < cap ? rpc : cap;
 }
 
+// Axes past the reach of the samplers' floor by addition (kFloorMagic): the
+// scoring and gradient calls take their group-per-pose kernels, which floor
+// with floorf, whatever the number of poses.
+bool big_axes(const ligen_grid_t* g) { return dock_big(make_view(g, nullptr, 0.f)); }
+
 // Multiprocessors of the current device, asked once per device.
 int sm_count(int* out) {
   static std::atomic<int> known[64];
@@ -842,7 +847,7 @@ std::string score_key(const ScoreArgs& b, const int32_t* d_list, const int* used
 // call's largest ligand) and replayed from a cached CUDA graph, or in one
 // group-per-pose launch.
 int run_score(const ScoreArgs& base, const ScorePlan& sp, const int32_t* d_list, cudaStream_t s) {
-  if (base.P < kLanePosesMin) {   // reads the moving-atom lists
+  if (base.P < kLanePosesMin || dock_big(base.grid)) {   // reads the moving-atom lists
     if (!base.pk.frag) return fail(LIGEN_ERR_CUDA, "internal: scoring without the moving-atom lists");
     LG_CUDA(launch_score(base, s));
     return LIGEN_OK;
@@ -1414,7 +1419,8 @@ int ligen_score_poses(const ligen_ligands_t* ligands, const ligen_grid_t* grid, 
   const size_t pose_floats = (size_t)poses_per_ligand * (7 * (size_t)L + sh.rot);
   const size_t nscores = (size_t)poses_per_ligand * L;
   ScorePlan plan;
-  if (poses_per_ligand >= kLanePosesMin) plan_score(ligands->h_rot_off, L, &plan);   // pose-per-lane launches
+  const bool lanes = poses_per_ligand >= kLanePosesMin && !big_axes(grid);
+  if (lanes) plan_score(ligands->h_rot_off, L, &plan);   // pose-per-lane launches
   Arena ar;
   LigandPlan lp;
   plan_ligands(ar, ligands, sh, lhost == 1, &lp);
@@ -1422,7 +1428,6 @@ int ligen_score_poses(const ligen_ligands_t* ligands, const ligen_grid_t* grid, 
   const size_t o_coef = ar.take(grid_coef_bytes(grid));
   const size_t o_xc = ar.take(16 * (size_t)sh.atoms);
   const size_t o_binfo = ar.take(4 * (size_t)sh.rot);
-  const bool lanes = poses_per_ligand >= kLanePosesMin;
   const size_t o_frag = lanes ? 0 : ar.take((size_t)kFragStride * sh.rot);   // the table replaces the lists
   const size_t o_status = ar.take(4 * (size_t)L);
   const size_t o_list = ar.take(4 * plan.list.size());
@@ -1682,7 +1687,7 @@ static int grad_call(const ligen_ligands_t* ligands, const ligen_grid_t* grid, i
   const size_t o_coef = ar.take(grid_coef_bytes(grid));
   const size_t o_xc = ar.take(16 * (size_t)sh.atoms);
   const size_t o_binfo = ar.take(4 * (size_t)sh.rot);
-  const bool lanes = poses_per_ligand >= kGradLanePosesMin;
+  const bool lanes = poses_per_ligand >= kGradLanePosesMin && !big_axes(grid);
   const size_t o_frag = lanes ? 0 : ar.take((size_t)kFragStride * sh.rot);   // the table replaces the lists
   const size_t o_status = ar.take(4 * (size_t)L);
   ScorePlan plan;   // ligands by rotatable-bond class for the pose-group kernel
