@@ -353,10 +353,12 @@ def _pose_lengths(ligands: Ligands, poses_per_ligand: int, device) -> torch.Tens
 
 
 def _kernel_reads(t: torch.Tensor) -> bool:
-    """Whether t's memory is all there is to it: no graph to extend, no vmap
-    level, no forward-mode tangent, no subclass, no dispatch mode watching."""
+    """Whether t's memory is all there is to it: no graph to extend, no lazy
+    negation, no zeros without storage, no vmap level, no forward-mode tangent,
+    no subclass, no dispatch mode watching."""
     return (type(t) is torch.Tensor and not (torch.is_grad_enabled() and t.requires_grad)
-            and torch._C._has_storage(t) and not torch._C._functorch.is_functorch_wrapped_tensor(t)
+            and torch._C._has_storage(t) and not t.is_neg() and not t._is_zerotensor()
+            and not torch._C._functorch.is_functorch_wrapped_tensor(t)
             and forward_ad._current_level < 0
             and torch._C._len_torch_dispatch_stack() == 0)
 
@@ -377,7 +379,7 @@ class PoseScore(torch.autograd.Function):
         ligands, grid, P, pen = ctx.args
         if _kernel_reads(grad_scores):   # the kernel multiplies each pose's gradient by its score's
             return _weighted_pose_grad(ligands, grid, poses.detach().contiguous(), P, pen, grad_scores), None, None, None, None
-        # create_graph, vmap (is_grads_batched), forward mode: torch multiplies
+        # create_graph, lazy bits, vmap (is_grads_batched), forward mode: torch multiplies
         _, grads = pose_grad(ligands, grid, poses.detach().contiguous(), P, pen)
         weight = grad_scores.reshape(-1).repeat_interleave(_pose_lengths(ligands, P, poses.device))
         return grads * weight, None, None, None, None
