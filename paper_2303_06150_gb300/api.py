@@ -355,12 +355,16 @@ def _pose_lengths(ligands: Ligands, poses_per_ligand: int, device) -> torch.Tens
 def _kernel_reads(t: torch.Tensor) -> bool:
     """Whether t's memory is all there is to it: no graph to extend, no lazy
     negation, no zeros without storage, no vmap level, no forward-mode tangent,
-    no subclass, no dispatch mode watching."""
-    return (type(t) is torch.Tensor and not (torch.is_grad_enabled() and t.requires_grad)
-            and torch._C._has_storage(t) and not t.is_neg() and not t._is_zerotensor()
-            and not torch._C._functorch.is_functorch_wrapped_tensor(t)
-            and forward_ad._current_level < 0
-            and torch._C._len_torch_dispatch_stack() == 0)
+    no subclass, no dispatch mode watching. Torch has no public name for some
+    of these questions; a version without one of the private names answers no."""
+    try:
+        return (type(t) is torch.Tensor and not (torch.is_grad_enabled() and t.requires_grad)
+                and torch._C._has_storage(t) and not t.is_neg() and not t._is_zerotensor()
+                and not torch._C._functorch.is_functorch_wrapped_tensor(t)
+                and forward_ad._current_level < 0
+                and torch._C._len_torch_dispatch_stack() == 0)
+    except AttributeError:
+        return False
 
 
 class PoseScore(torch.autograd.Function):
