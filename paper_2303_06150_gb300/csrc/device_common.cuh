@@ -193,9 +193,17 @@ __device__ __forceinline__ bool lg_check(unsigned* check, bool ok, unsigned code
 }
 
 // Index (in records) of the record of channel c, cell (ix, iy, iz); the
-// grid preparation writes records at the same indices.
+// grid preparation writes records at the same indices. A channel of 16-bit
+// records can hold more than 2^31 cells: an accepted grid has at most 2e9
+// cells times channels, the records' padding (rec_cells) multiplies a thin
+// grid's by up to 8.
 __host__ __device__ __forceinline__ size_t rec_index(int cx, int cy, int cz, int c, int ix, int iy, int iz) {
-  return (size_t)c * cz * cy * cx + (size_t)((iz * cy + iy) * cx + ix);
+  return (size_t)c * cz * cy * cx + ((size_t)iz * cy + iy) * cx + ix;
+}
+// The same for coefficient records, which have no padding: a channel's at
+// most 2e9 cells are counted in 32 bits.
+__host__ __device__ __forceinline__ size_t rec_index_f32(int cx, int cy, int cz, int c, int ix, int iy, int iz) {
+  return (size_t)c * cz * cy * cx + (unsigned)((iz * cy + iy) * cx + ix);
 }
 // Records to allocate for a grid of cx * cy * cz cells and nc channels.
 __host__ __device__ __forceinline__ size_t rec_count(int cx, int cy, int cz, int nc) {
@@ -259,7 +267,7 @@ __device__ __forceinline__ float grid_sample(const GridView& g, float ux, float 
     float fz = fminf(floorf(uz), g.mz - 1.f);
     int ix = (int)fx, iy = (int)fy, iz = (int)fz;
     float dx = ux - fx, dy = uy - fy, dz = uz - fz;
-    const size_t ri = rec_index(g.cx, g.cy, g.cz, c, ix, iy, iz);
+    const size_t ri = rec_index_f32(g.cx, g.cy, g.cz, c, ix, iy, iz);
     if (!lg_check(g.check, c >= 0 && c < g.nc && ri < g.n_rec, kChkGridRecord)) return g.penalty;
     const float* rec = g.coef + ri * 8;
     float a[8];
@@ -366,9 +374,11 @@ __device__ __forceinline__ float grid_sample_fmt(const GridView& g, float ux, fl
 //             and NaN above every coordinate of the box: one comparison per
 //             axis. A coordinate of -0 would count as outside; positions here
 //             are sums that start from t - origin, which is never -0;
-//   record    32-bit index arithmetic on the unreduced bits, their constant
-//             part subtracted once (GridView::bias). Bounds, bias and cell
-//             counts are constant-bank operands: none takes a register.
+//   record    32-bit index arithmetic (no axis has 2^23 cells here, so a
+//             channel has fewer than 2^32, padding included) on the
+//             unreduced bits, their constant part subtracted once
+//             (GridView::bias). Bounds, bias and cell counts are
+//             constant-bank operands: none takes a register.
 //
 // Measured on GB300 against floorf, conversions, six comparisons and a clamp
 // per scalar sample (docking kernel, 12,000 screening / 3,000 bimodal
@@ -467,7 +477,7 @@ __device__ __forceinline__ float grid_sample_grad(const GridView& g, float ux, f
     float fz = fminf(floorf(uz), g.mz - 1.f);
     int ix = (int)fx, iy = (int)fy, iz = (int)fz;
     float dx = ux - fx, dy = uy - fy, dz = uz - fz;
-    const size_t ri = rec_index(g.cx, g.cy, g.cz, c, ix, iy, iz);
+    const size_t ri = rec_index_f32(g.cx, g.cy, g.cz, c, ix, iy, iz);
     if (!lg_check(g.check, c >= 0 && c < g.nc && ri < g.n_rec, kChkGridRecord)) return g.penalty;
     const float* rec = g.coef + ri * 8;
     float a[8];
