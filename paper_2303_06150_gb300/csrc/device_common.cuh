@@ -1,6 +1,7 @@
 // Device building blocks shared by the docking kernels: the restart random
 // stream, quaternion algebra, the cube rotation table and the grid sampler.
 #pragma once
+#include <cmath>
 #include <cstdint>
 #include <cuda_bf16.h>
 #include <cuda_fp16.h>
@@ -159,7 +160,8 @@ struct GridView {
   const float* coef;   // records at rec_index, 256-byte aligned
   int cx, cy, cz;      // record cells per axis (rec_cells of the format)
   int nc;
-  float mx, my, mz;    // points - 1 per axis, as float: upper box bound in grid units
+  float mx, my, mz;    // points - 1 per axis: upper box bound in grid units (axis_bounds)
+  float kx, ky, kz;    // points - 2: the last cell of FP32 records
   // operands of the docking kernel's sampler (DockPoint)
   float lx, ly, lz;    // the floats below mx, my, mz
   unsigned hx, hy, hz; // bits of mx, my, mz
@@ -169,6 +171,18 @@ struct GridView {
   size_t n_rec;        // records in the buffer (checked builds compare with it)
   unsigned* check;     // checked builds: first out-of-range code, else NULL
 };
+
+// The upper box bound and the last cell of an axis of n points as floats,
+// rounded towards zero: past 2^24 points the nearest float can lie beyond the
+// last point, and a coordinate there would be given a cell past the records.
+inline void axis_bounds(int n, float* top, float* last_cell) {
+  auto below = [](int v) {
+    const float f = (float)v;
+    return (double)f > (double)v ? std::nextafterf(f, 0.f) : f;
+  };
+  *top = below(n - 1);
+  *last_cell = below(n - 2);
+}
 
 // Checked builds (compiled with -DLIGEN_CHECKED=1): every data-dependent
 // index is compared with its bound before use; a violation stores its code
@@ -262,9 +276,9 @@ __device__ __forceinline__ float grid_sample(const GridView& g, float ux, float 
   bool inb = (ux >= 0.f) & (ux <= g.mx) & (uy >= 0.f) & (uy <= g.my) & (uz >= 0.f) & (uz <= g.mz);
   float e = g.penalty;
   if (inb) {
-    float fx = fminf(floorf(ux), g.mx - 1.f);
-    float fy = fminf(floorf(uy), g.my - 1.f);
-    float fz = fminf(floorf(uz), g.mz - 1.f);
+    float fx = fminf(floorf(ux), g.kx);
+    float fy = fminf(floorf(uy), g.ky);
+    float fz = fminf(floorf(uz), g.kz);
     int ix = (int)fx, iy = (int)fy, iz = (int)fz;
     float dx = ux - fx, dy = uy - fy, dz = uz - fz;
     const size_t ri = rec_index_f32(g.cx, g.cy, g.cz, c, ix, iy, iz);
@@ -472,9 +486,9 @@ __device__ __forceinline__ float grid_sample_grad(const GridView& g, float ux, f
   float e = g.penalty;
   *gx = *gy = *gz = 0.f;
   if (inb) {
-    float fx = fminf(floorf(ux), g.mx - 1.f);
-    float fy = fminf(floorf(uy), g.my - 1.f);
-    float fz = fminf(floorf(uz), g.mz - 1.f);
+    float fx = fminf(floorf(ux), g.kx);
+    float fy = fminf(floorf(uy), g.ky);
+    float fz = fminf(floorf(uz), g.kz);
     int ix = (int)fx, iy = (int)fy, iz = (int)fz;
     float dx = ux - fx, dy = uy - fy, dz = uz - fz;
     const size_t ri = rec_index_f32(g.cx, g.cy, g.cz, c, ix, iy, iz);

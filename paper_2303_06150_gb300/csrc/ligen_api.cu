@@ -293,7 +293,9 @@ GridView make_view(const ligen_grid_t* g, const float* coef, float penalty, int 
   v.n_rec = rec_count(v.cx, v.cy, v.cz, g->nc);
   v.check = nullptr;
   v.nc = g->nc;
-  v.mx = (float)(g->nx - 1); v.my = (float)(g->ny - 1); v.mz = (float)(g->nz - 1);
+  axis_bounds(g->nx, &v.mx, &v.kx);
+  axis_bounds(g->ny, &v.my, &v.ky);
+  axis_bounds(g->nz, &v.mz, &v.kz);
   v.lx = std::nextafterf(v.mx, 0.f); v.ly = std::nextafterf(v.my, 0.f); v.lz = std::nextafterf(v.mz, 0.f);
   auto bits = [](float f) {
     unsigned b;
