@@ -3,13 +3,15 @@
 // values in 16 bits), at rec_index (channel-major, see GridView).
 //
 // The bound is the write of the records (96^3 x 8 nodes: 219 MB in FP32
-// against 28 MB read). A thread owns one (x, channel) column of a row of
-// cells and marches along z, so a cell's lower corners are the registers of
-// the cell below and every step costs four loads (consecutive threads:
-// consecutive channels, then x; whole lines), twelve additions and one store
-// of the whole record; indices are divided out once per thread. Measured on
-// GB300, 96^3 x 8: FP32 63 -> 40.5 us (6.1 TB/s), FP16 66 -> 35 us, against
-// one thread per record with 64-bit divisions and eight loads each.
+// against 28 MB read). A thread owns one (x, y, channel) column of cells and
+// marches along z, so a cell's lower corners are the registers of the cell
+// below and every step costs four loads (consecutive threads: consecutive
+// channels, then x, then y; whole lines, and no idle threads however short a
+// row is), twelve additions and one store of the whole record; indices are
+// divided out once per thread. Measured on GB300, 96^3 x 8: FP32 63 -> 40.5 us
+// (6.1 TB/s), FP16 66 -> 35 us, against one thread per record with 64-bit
+// divisions and eight loads each. With a block's threads inside one row, a
+// call with a 2 x 1500 x 1500 x 1 grid took 179 us, now 25.
 #include "internal.h"
 
 namespace ligen {
@@ -40,19 +42,20 @@ __device__ __forceinline__ unsigned pack16(float a, float b) {   // rounded to n
   }
 }
 
-// Block: (tile of the row's (x, channel) columns, row iy, march). 16-bit
+// Block: (tile of the plane's (x, y, channel) columns, march). 16-bit
 // record grids have rec_cells(n) = n cells per axis: corners past the last
 // node repeat it (the padding layers of the clamp-free sampler).
 template <int FMT>
 __global__ void __launch_bounds__(kPrepThreads) grid_prep_kernel(const float* __restrict__ v, int nx, int ny, int nz,
-                                                                 int nc, int tiles, int march,
+                                                                 int nc, unsigned tiles, int march,
                                                                  void* __restrict__ out) {
   const int cx = rec_cells(nx, FMT), cy = rec_cells(ny, FMT), cz = rec_cells(nz, FMT);
-  const unsigned tile = blockIdx.x % tiles, row = blockIdx.x / tiles;
-  const int iy = (int)(row % cy), z0 = (int)(row / cy) * march;
-  const unsigned t = tile * kPrepThreads + threadIdx.x;
-  if (t >= (unsigned)cx * nc) return;
-  const int ix = (int)(t / nc), c = (int)(t % nc);
+  const unsigned tile = blockIdx.x % tiles, t = tile * kPrepThreads + threadIdx.x;   // < 2^32 (check_grid)
+  const int z0 = (int)(blockIdx.x / tiles) * march;
+  const unsigned row = (unsigned)cx * nc;
+  const int iy = (int)(t / row);
+  if (iy >= cy) return;
+  const int ix = (int)(t % row / nc), c = (int)(t % row % nc);
   const int z1 = min(z0 + march, cz);
   const int x1 = FMT == kRecF32 ? ix + 1 : min(ix + 1, nx - 1), y1 = FMT == kRecF32 ? iy + 1 : min(iy + 1, ny - 1);
   const size_t plane = (size_t)nx * ny * nc;
@@ -93,10 +96,10 @@ template <int FMT>
 cudaError_t launch_prep(const float* values, int nx, int ny, int nz, int nc, void* rec, bool beside_pack,
                         cudaStream_t s) {
   const size_t cx = rec_cells(nx, FMT), cy = rec_cells(ny, FMT), cz = rec_cells(nz, FMT);
-  const size_t tiles = (cx * nc + kPrepThreads - 1) / kPrepThreads;
-  const size_t full = tiles * cy * cz / kPrepBlocks;
+  const size_t tiles = (cx * cy * nc + kPrepThreads - 1) / kPrepThreads;
+  const size_t full = tiles * cz / kPrepBlocks;
   const size_t march = full < 2 ? 2 : full < kPrepMarch ? full : kPrepMarch;
-  const size_t blocks = tiles * cy * ((cz + march - 1) / march);
+  const size_t blocks = tiles * ((cz + march - 1) / march);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)blocks);
   cfg.blockDim = dim3(kPrepThreads);
@@ -106,7 +109,7 @@ cudaError_t launch_prep(const float* values, int nx, int ny, int nz, int nc, voi
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = beside_pack ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, grid_prep_kernel<FMT>, values, nx, ny, nz, nc, (int)tiles, (int)march, rec);
+  return cudaLaunchKernelEx(&cfg, grid_prep_kernel<FMT>, values, nx, ny, nz, nc, (unsigned)tiles, (int)march, rec);
 }
 
 }  // namespace
