@@ -82,7 +82,13 @@ struct DockArgs {
 // and kExMaxCombos combinations (n_rigid * n_theta^n) per restart.
 constexpr int kExMaxRot = 4;
 constexpr long long kExMaxCombos = 1ll << 27;
-cudaError_t launch_exhaustive(const DockArgs& a, cudaStream_t s);
+// The largest ligand's table and chain: atoms times combinations of torsion
+// increments, atoms times their square root.
+struct ExWork {
+  long long entries = 0;
+  double chain = 0.;
+};
+cudaError_t launch_exhaustive(const DockArgs& a, const ExWork& w, int sms, cudaStream_t s);
 
 struct TopkArgs {
   int L, R, K, step_deg;

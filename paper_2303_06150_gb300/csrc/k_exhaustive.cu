@@ -18,13 +18,15 @@
 // the ones that do not fit (many increments, deeply nested bonds) are
 // rebuilt per combination.
 //
-// A cluster of kExCluster CTAs takes one (ligand, restart), the rotations
+// A cluster of 1, 2, 4 or 8 CTAs takes one (ligand, restart), the rotations
 // split over its CTAs, and joins its winners through distributed shared
 // memory: without the split a call of a few hundred restarts leaves the
-// chip to the few ligands with the most bonds.
+// chip to the few ligands with the most bonds, with it every CTA more stages
+// the ligand and lays out the table again. launch_exhaustive has the rule.
 // Measured on GB300, 97 ligands of 8-20 atoms and 0-3 bonds, 8 restarts, 30
 // degree steps, whole call: 2,780 us with every combination rebuilt by one
-// CTA per (ligand, restart), 242 us this way.
+// CTA per (ligand, restart), 269 us this way (280 with eight CTAs for every
+// call).
 #include <cooperative_groups.h>
 
 #include "../../include/ligen.h"
@@ -34,8 +36,9 @@ namespace ligen {
 namespace {
 
 constexpr int kExThreads = 128;
-constexpr int kExCluster = 8;     // CTAs per (ligand, restart): the portable maximum
-constexpr int kExTable = 6144;    // table entries: 24 KB, seven CTAs per SM with the rest
+constexpr int kExCluster = 8;     // CTAs per (ligand, restart), at most: the portable maximum
+constexpr int kExTable = 6144;    // table entries: 24 KB
+constexpr int kExSmall = 1024;    // table entries of the build for little work
 constexpr int kExVec = 4;         // combinations a thread sums side by side
 constexpr uint16_t kExDirect = 0xffffu;
 
@@ -45,19 +48,30 @@ constexpr uint16_t kExDirect = 0xffffu;
 struct ExDiv {
   unsigned d;
   unsigned long long m;
-  __device__ explicit ExDiv(unsigned dd) : d(dd), m(((1ull << 40) + dd - 1) / dd) {}
+  explicit ExDiv(unsigned dd) : d(dd), m(((1ull << 40) + dd - 1) / dd) {}
   __device__ unsigned operator()(unsigned q) const { return d == 1 ? q : (unsigned)((q * m) >> 40); }
 };
 
+// A launch: CTAs per (ligand, restart), table entries per CTA, atoms of the
+// largest ligand rounded up to 16.
+struct ExLaunch {
+  int cluster, table, acap;
+  ExDiv by_nt;
+};
+
+// Shared memory for ligands of at most acap atoms (a multiple of 16), the
+// table behind them.
 struct ExLigand {
-  float4 sx[LIGEN_MAX_ATOMS];
-  uint2 stride[LIGEN_MAX_ATOMS];    // table strides of bonds 0..3, 16 bits each
-  uint16_t base[LIGEN_MAX_ATOMS];   // first table entry, or kExDirect
-  uint8_t mask[LIGEN_MAX_ATOMS];    // bonds that move the atom
-  uint8_t slot[LIGEN_MAX_ATOMS];    // tabled atoms by first entry
-  int axis[kExMaxRot][2];
+  float4* sx;
+  uint2* stride;     // table strides of bonds 0..3, 16 bits each
+  uint16_t* base;    // first table entry, or kExDirect
+  uint8_t* mask;     // bonds that move the atom
+  uint8_t* slot;     // tabled atoms by first entry
+  float* tab;
+  int (*axis)[2];    // [kExMaxRot]
   int n_slots, entries;
 };
+__host__ __device__ inline size_t ex_smem_bytes(int acap, int table) { return 28 * (size_t)acap + 4 * (size_t)table; }
 
 // Bond b's axis after the earlier bonds of `use` with increments j: moving
 // end pv, unit direction kd, and the turn's cosine and sine.
@@ -109,7 +123,7 @@ __device__ __forceinline__ float ex_energy(const DockArgs& a, const ExLigand& S,
 // Best of `total` combinations that start at combination c0 of the search
 // (whole rotations; the table holds them), all atoms tabled. NB >= n.
 template <int NB>
-__device__ __forceinline__ void ex_sum(const ExLigand& S, const float* tab, int N, int n, const ExDiv& by_nt,
+__device__ __forceinline__ void ex_sum(const ExLigand& S, int N, int n, const ExDiv& by_nt,
                                        unsigned total, long long c0, float& best, long long& bestc) {
   for (unsigned t = threadIdx.x; t < total; t += kExThreads * kExVec) {
     unsigned off[kExVec];
@@ -139,7 +153,7 @@ __device__ __forceinline__ void ex_sum(const ExLigand& S, const float* tab, int 
         if constexpr (NB > 1) at += j[v][1] * (s.x >> 16);
         if constexpr (NB > 2) at += j[v][2] * (s.y & 0xffffu);
         if constexpr (NB > 3) at += j[v][3] * (s.y >> 16);
-        acc[v] -= tab[at];
+        acc[v] -= S.tab[at];
       }
     }
 #pragma unroll
@@ -151,27 +165,38 @@ __device__ __forceinline__ void ex_sum(const ExLigand& S, const float* tab, int 
   }
 }
 
-template <int FMT>
-__global__ void __cluster_dims__(kExCluster, 1, 1) __launch_bounds__(kExThreads)
-    exhaustive_kernel(const DockArgs a, long long first) {
+// MINB: resident CTAs asked of the register allocator: 1 (155 registers, three
+// CTAs per SM), or 8 (64, spilling) for launches of little work, whose time is
+// what every CTA does before and after it.
+template <int FMT, int MINB>
+__global__ void __launch_bounds__(kExThreads, MINB) exhaustive_kernel(const DockArgs a, const ExLaunch x, unsigned first) {
   namespace cg = cooperative_groups;
-  __shared__ ExLigand S;
-  __shared__ float tab[kExTable];
+  extern __shared__ __align__(16) unsigned char ex_smem[];
+  __shared__ int s_axis[kExMaxRot][2];
+  __shared__ int s_table[2];   // tabled atoms, entries
   __shared__ float red_s[kExThreads / 32];
   __shared__ long long red_c[kExThreads / 32];
   __shared__ float cta_s;
   __shared__ long long cta_c;
 
-  const long long item = first + blockIdx.x / kExCluster;
-  const int rank = blockIdx.x % kExCluster;
-  const int l = (int)(item / a.R), r = (int)(item % a.R);
+  ExLigand S;
+  S.sx = reinterpret_cast<float4*>(ex_smem);
+  S.stride = reinterpret_cast<uint2*>(S.sx + x.acap);
+  S.tab = reinterpret_cast<float*>(S.stride + x.acap);
+  S.base = reinterpret_cast<uint16_t*>(S.tab + x.table);
+  S.mask = reinterpret_cast<uint8_t*>(S.base + x.acap);
+  S.slot = S.mask + x.acap;
+  S.axis = s_axis;
+  const unsigned item = first + blockIdx.x / (unsigned)x.cluster;   // < 2^31 (checked on the host)
+  const int rank = (int)(blockIdx.x % (unsigned)x.cluster);
+  const int l = (int)(item / (unsigned)a.R), r = (int)(item % (unsigned)a.R);
   if (a.pk.status[l] != 0) return;   // uniform over the cluster
   const int tid = threadIdx.x;
   const int a0 = a.lig.atom_off[l];
   const int N = a.lig.atom_off[l + 1] - a0;
   const int r0 = a.lig.rot_off[l];
   const int n = a.lig.rot_off[l + 1] - r0;   // <= kExMaxRot (checked on the host)
-  if (!lg_check(a.grid.check, N <= LIGEN_MAX_ATOMS && n <= kExMaxRot, kChkItemShape)) return;   // uniform
+  if (!lg_check(a.grid.check, N <= x.acap && n <= kExMaxRot, kChkItemShape)) return;   // uniform
 
   for (int i = tid; i < N; i += kExThreads) {
     S.sx[i] = a.pk.xc[a0 + i];
@@ -193,39 +218,44 @@ __global__ void __cluster_dims__(kExCluster, 1, 1) __launch_bounds__(kExThreads)
     __syncthreads();
   }
   // table layout for one rotation: atoms by ascending count of bonds, then by index
-  const unsigned nt = (unsigned)a.n_theta;
+  const unsigned nt = x.by_nt.d;
   if (tid < 32) {
-    int used = 0, slots = 0;
-    long long size = 1;
-    for (int m = 0; m <= n; ++m, size *= nt)
+    unsigned used = 0, slots = 0, size = 1;   // entries of an atom moved by m bonds; past the table: any larger value
+    for (int m = 0; m <= n; ++m) {
+      const unsigned room = size <= (unsigned)x.table ? (x.table - used) / size : 0u;
+      unsigned seen = 0;
       for (int w = 0; w < N; w += 32) {
         const int i = w + tid;
         const bool in = i < N && __popc(S.mask[i < N ? i : 0]) == m;
         const unsigned all = __ballot_sync(0xffffffffu, in);
-        const int before = __popc(all & ((1u << tid) - 1u));
-        const long long fit = (kExTable - used) / size;
+        const unsigned at = seen + __popc(all & ((1u << tid) - 1u));
         if (in) {
-          const bool tabled = before < fit;
+          const bool tabled = at < room;
           unsigned st[kExMaxRot] = {0u, 0u, 0u, 0u};
           if (tabled) {
             unsigned s = 1u;
             for (int b = n - 1; b >= 0; --b)
               if (S.mask[i] >> b & 1u) { st[b] = s; s *= nt; }
-            S.slot[slots + before] = (uint8_t)i;
+            S.slot[slots + at] = (uint8_t)i;
           }
           S.stride[i] = make_uint2(st[0] | st[1] << 16, st[2] | st[3] << 16);
-          S.base[i] = tabled ? (uint16_t)(used + before * size) : kExDirect;
+          S.base[i] = tabled ? (uint16_t)(used + at * size) : kExDirect;
         }
-        const int kept = (int)(__popc(all) < fit ? __popc(all) : fit);
-        used += (int)(kept * size);
-        slots += kept;
+        seen += __popc(all);
       }
+      const unsigned kept = min(seen, room);
+      used += kept * size;
+      slots += kept;
+      size = min(size * nt, (unsigned)kExTable + 1u);
+    }
     if (tid == 0) {
-      S.entries = used;
-      S.n_slots = slots;
+      s_table[0] = (int)slots;
+      s_table[1] = (int)used;
     }
   }
   __syncthreads();
+  S.n_slots = s_table[0];
+  S.entries = s_table[1];
 
   // restart orientation and translation, as in the greedy kernel
   float u[6];
@@ -243,11 +273,11 @@ __global__ void __cluster_dims__(kExCluster, 1, 1) __launch_bounds__(kExThreads)
     o[k] = (t - a.origin[k]) * a.inv_h;
   }
 
-  const ExDiv by_nt(nt);
+  const ExDiv& by_nt = x.by_nt;
   unsigned per_k = 1;   // <= 2^27 (checked on the host)
   for (int b = 0; b < n; ++b) per_k *= nt;
-  const int k_lo = a.n_rigid * rank / kExCluster, k_hi = a.n_rigid * (rank + 1) / kExCluster;
-  const int batch = S.entries ? max(1, kExTable / S.entries) : k_hi - k_lo;   // rotations tabled together
+  const int k_lo = a.n_rigid * rank / x.cluster, k_hi = a.n_rigid * (rank + 1) / x.cluster;
+  const int batch = S.entries ? max(1, x.table / S.entries) : k_hi - k_lo;   // rotations tabled together
   float best = -INFINITY;
   long long bestc = 0x7fffffffffffffffll;
   for (int k0 = k_lo; k0 < k_hi; k0 += batch) {
@@ -278,16 +308,16 @@ __global__ void __cluster_dims__(kExCluster, 1, 1) __launch_bounds__(kExThreads)
       float G[9], Mk[9];
       cube_mat(k0 + kk, G);
       mat3mul(M, G, Mk);
-      tab[e] = ex_energy<FMT>(a, S, i, n, Mk, o, pv, kd, cs, sn);
+      S.tab[e] = ex_energy<FMT>(a, S, i, n, Mk, o, pv, kd, cs, sn);
     }
     __syncthreads();
     const unsigned total = per_k * (unsigned)nk;
     const long long c0 = (long long)k0 * per_k;
     if (S.n_slots == N) {
-      if (n <= 1) ex_sum<1>(S, tab, N, n, by_nt, total, c0, best, bestc);
-      else if (n == 2) ex_sum<2>(S, tab, N, n, by_nt, total, c0, best, bestc);
-      else if (n == 3) ex_sum<3>(S, tab, N, n, by_nt, total, c0, best, bestc);
-      else ex_sum<4>(S, tab, N, n, by_nt, total, c0, best, bestc);
+      if (n <= 1) ex_sum<1>(S, N, n, by_nt, total, c0, best, bestc);
+      else if (n == 2) ex_sum<2>(S, N, n, by_nt, total, c0, best, bestc);
+      else if (n == 3) ex_sum<3>(S, N, n, by_nt, total, c0, best, bestc);
+      else ex_sum<4>(S, N, n, by_nt, total, c0, best, bestc);
     } else {
       for (unsigned t = tid; t < total; t += kExThreads) {
         unsigned q = t;
@@ -310,7 +340,7 @@ __global__ void __cluster_dims__(kExCluster, 1, 1) __launch_bounds__(kExThreads)
         for (int i = 0; i < N; ++i) {
           if (S.base[i] != kExDirect) {   // uniform
             const uint2 s = S.stride[i];
-            acc -= tab[S.base[i] + q * S.entries + j[0] * (s.x & 0xffffu) + j[1] * (s.x >> 16) +
+            acc -= S.tab[S.base[i] + q * S.entries + j[0] * (s.x & 0xffffu) + j[1] * (s.x >> 16) +
                        j[2] * (s.y & 0xffffu) + j[3] * (s.y >> 16)];
           } else {
             acc -= ex_energy<FMT>(a, S, i, n, Mk, o, pv, kd, cs, sn);
@@ -337,9 +367,9 @@ __global__ void __cluster_dims__(kExCluster, 1, 1) __launch_bounds__(kExThreads)
     cta_c = bestc;
   }
   cg::cluster_group cluster = cg::this_cluster();
-  cluster.sync();
+  if (x.cluster > 1) cluster.sync();
   if (rank == 0 && tid == 0) {
-    for (int c = 1; c < kExCluster; ++c) {
+    for (int c = 1; c < x.cluster; ++c) {
       const float os = *cluster.map_shared_rank(&cta_s, c);
       const long long oc = *cluster.map_shared_rank(&cta_c, c);
       if (os > best || (os == best && oc < bestc)) { best = os; bestc = oc; }
@@ -354,20 +384,58 @@ __global__ void __cluster_dims__(kExCluster, 1, 1) __launch_bounds__(kExThreads)
     for (int b = n - 1; b >= 0; --b) { cnt[b] = (uint8_t)(rem % nt); rem /= nt; }
     a.res_k[lr] = (uint8_t)rem;
   }
-  cluster.sync();   // the other CTAs' winners stay readable until here
+  if (x.cluster > 1) cluster.sync();   // the other CTAs' winners stay readable until here
 }
 
 }  // namespace
 
-cudaError_t launch_exhaustive(const DockArgs& a, cudaStream_t s) {
-  const auto kernel = a.fmt == kRecF32   ? exhaustive_kernel<kRecF32>
-                      : a.fmt == kRecF16 ? exhaustive_kernel<kRecF16>
-                                         : exhaustive_kernel<kRecBF16>;
-  const long long items = (long long)a.lig.L * a.R, most = (1ll << 31) / kExCluster - 1;   // grid limit
+// The CTAs of a (ligand, restart) and the build. Each of items * C CTAs costs
+// about 5.6 us of a slot (3 per SM) before and after its work, so C of them
+// lengthen the launch by a C; the chain of the largest ligand's rotations
+// shortens it to b / C, at about 14 ns per rotation, atom and square root of
+// its combinations (an atom's table entries lie between 1 and all
+// combinations; the geometric mean). The C with the smallest sum is taken,
+// no more than there are rotations. Where all rotations fit kExSmall entries
+// the chain is short whatever C. Measured on GB300, whole calls (us; 1,000,
+// 100, 50 or 5,000 ligands of 8-20 atoms, restarts, 30 degree steps, 24
+// rotations), * the one chosen; "rebuilt" is one CTA per (ligand, restart)
+// with every combination rebuilt:
+//                        rebuilt   C = 1     2       4       8     small build
+//   0 bonds   5,000 x 16     844    1,053   2,041   3,902   8,567     591*
+//   0-1       5,000 x 16   1,644    1,363*  2,534   4,680   9,806     984
+//   2         1,000 x 16   4,469      854*  1,078   1,564   2,705     846
+//   2         1,000 x 1      425      268     151*    141     199     473
+//   3         50 x 16      4,035      255     243     254*    331     312
+//   0-3       100 x 1      2,651      236     132      85      64*    404
+cudaError_t launch_exhaustive(const DockArgs& a, const ExWork& w, int sms, cudaStream_t s) {
+  const long long items = (long long)a.lig.L * a.R;
+  const bool small = w.entries * a.n_rigid <= kExSmall;
+  const double per_cta = 5.6 * (double)items / (3. * sms), chain = 0.014 * a.n_rigid * w.chain;
+  int C = 1;
+  for (int c = 2; c <= kExCluster && c <= a.n_rigid && !small; c *= 2)
+    if (per_cta * c + chain / c < per_cta * C + chain / C) C = c;
+  const auto kernel = small ? a.fmt == kRecF32   ? exhaustive_kernel<kRecF32, 8>
+                              : a.fmt == kRecF16 ? exhaustive_kernel<kRecF16, 8>
+                                                 : exhaustive_kernel<kRecBF16, 8>
+                      : a.fmt == kRecF32   ? exhaustive_kernel<kRecF32, 1>
+                        : a.fmt == kRecF16 ? exhaustive_kernel<kRecF16, 1>
+                                           : exhaustive_kernel<kRecBF16, 1>;
+  const ExLaunch x{C, small ? kExSmall : kExTable, (a.max_atoms + 15) / 16 * 16, ExDiv((unsigned)a.n_theta)};
+  const long long most = (1ll << 31) / C - 1;   // grid limit
   for (long long first = 0; first < items; first += most) {
     const long long here = items - first < most ? items - first : most;
-    kernel<<<(unsigned)(here * kExCluster), kExThreads, 0, s>>>(a, first);
-    const cudaError_t e = cudaGetLastError();
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)(here * C));
+    cfg.blockDim = dim3(kExThreads);
+    cfg.dynamicSmemBytes = ex_smem_bytes(x.acap, x.table);   // <= 32 KB
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeClusterDimension;
+    at.val.clusterDim.x = (unsigned)C;
+    at.val.clusterDim.y = at.val.clusterDim.z = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = C > 1 ? 1 : 0;
+    const cudaError_t e = cudaLaunchKernelEx(&cfg, kernel, a, x, (unsigned)first);
     if (e != cudaSuccess) return e;
   }
   return cudaSuccess;

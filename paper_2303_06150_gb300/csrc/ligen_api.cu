@@ -214,22 +214,29 @@ int check_params(const ligen_params_t* p) {
 }
 
 // Exhaustive mode: small ligands only (see ligen_params_t.mode).
-int check_exhaustive(const ligen_ligands_t* g, const ligen_params_t* p) {
+int check_exhaustive(const ligen_ligands_t* g, const ligen_params_t* p, ExWork* work) {
   if (p->trace) return fail(LIGEN_ERR_INVALID_ARG, "trace is not written in exhaustive mode (mode 1)");
   if (p->coords) return fail(LIGEN_ERR_INVALID_ARG, "coords are not written in exhaustive mode (mode 1)");
   if ((int64_t)g->n_ligands * p->restarts > INT32_MAX)
     return fail(LIGEN_ERR_UNSUPPORTED, "exhaustive mode: ligands * restarts exceeds 2^31 - 1");
   const int nt = 360 / p->torsion_step_deg;
+  long long combos_of[kExMaxRot + 1] = {1};   // of the torsion increments, by bonds
+  double root_of[kExMaxRot + 1] = {1.};
+  for (int n = 1; n <= kExMaxRot; ++n) {
+    combos_of[n] = combos_of[n - 1] * nt;
+    root_of[n] = std::sqrt((double)combos_of[n]);
+  }
   for (int l = 0; l < g->n_ligands; ++l) {
-    const int n = g->h_rot_off[l + 1] - g->h_rot_off[l];
+    const int n = g->h_rot_off[l + 1] - g->h_rot_off[l], N = g->h_atom_off[l + 1] - g->h_atom_off[l];
     if (n > kExMaxRot)
       return fail(LIGEN_ERR_UNSUPPORTED, "exhaustive mode: ligand %d has %d rotatable bonds (max %d)", l, n,
                   kExMaxRot);
-    long long combos = p->n_rigid;
-    for (int b = 0; b < n; ++b) combos *= nt;
+    const long long combos = p->n_rigid * combos_of[n];
     if (combos > kExMaxCombos)
       return fail(LIGEN_ERR_UNSUPPORTED, "exhaustive mode: ligand %d needs %lld poses per restart (max %lld)", l,
                   combos, kExMaxCombos);
+    work->entries = std::max(work->entries, N * combos_of[n]);
+    work->chain = std::max(work->chain, N * root_of[n]);
   }
   return LIGEN_OK;
 }
@@ -990,7 +997,8 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
   cudaStream_t s = (cudaStream_t)params->stream;
   const int R = params->restarts, K = params->top_k, P = params->passes;
   const bool exhaustive = params->mode == 1;
-  if (exhaustive && (rc = check_exhaustive(ligands, params)) != LIGEN_OK) return rc;
+  ExWork ex_work;
+  if (exhaustive && (rc = check_exhaustive(ligands, params, &ex_work)) != LIGEN_OK) return rc;
 
   const int lhost = space_of({ligands->atom_off, ligands->xyz, ligands->type, ligands->bonds,
                               ligands->rot_off, ligands->rot_edge});
@@ -1067,8 +1075,8 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
   int sms = 0;
   int lanes = kDefaultLanes;
   bool longest_first = false;
+  if (!buckets && (rc = sm_count(&sms)) != LIGEN_OK) return rc;
   if (!buckets && !exhaustive) {
-    if ((rc = sm_count(&sms)) != LIGEN_OK) return rc;
     if (!any_big)
       lanes = dock_pick_lanes(ligands->h_atom_off, ligands->h_rot_off, L, R, params->n_rigid,
                               360 / params->torsion_step_deg, P, fmt, sms);
@@ -1217,7 +1225,7 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
     da.samples = d_samples;
     if (longest_first) da.list = ar.at<int32_t>(o_order);
     if (exhaustive) {
-      LG_CUDA(launch_exhaustive(da, st));
+      LG_CUDA(launch_exhaustive(da, ex_work, sms, st));
     } else if (buckets) {
       // Uploaded on every call: any other call on this stream may have
       // carved the workspace differently and overwritten this region (a

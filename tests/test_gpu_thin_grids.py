@@ -58,6 +58,6 @@ def test_short_rows_cost_no_more_than_long_ones():
             best = min(best, t[0].elapsed_time(t[1]) * 250)
         return best
 
-    # 4.0 M records; the rest of the call (packer, scoring, launches) is in both. With a row of cells to a block,
-    # 1500 for 2000 took 179 against 35 us; now 25 against 34
+    # 4.0 M records; the rest of the call (packer, scoring, launches) is in both. With a row of cells to a block:
+    # 369 against 44 us
     assert us(2, 2000, 2000) <= 2 * us(2000, 2000, 2)
