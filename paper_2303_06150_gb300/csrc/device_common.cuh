@@ -161,7 +161,6 @@ struct GridView {
   int cx, cy, cz;      // record cells per axis (rec_cells of the format)
   int nc;
   float mx, my, mz;    // points - 1 per axis: upper box bound in grid units (axis_bounds)
-  float kx, ky, kz;    // points - 2: the last cell of FP32 records
   // operands of the docking kernel's sampler (DockPoint)
   float lx, ly, lz;    // the floats below mx, my, mz
   unsigned hx, hy, hz; // bits of mx, my, mz
@@ -170,6 +169,11 @@ struct GridView {
   float penalty;
   size_t n_rec;        // records in the buffer (checked builds compare with it)
   unsigned* check;     // checked builds: first out-of-range code, else NULL
+  // points - 2: the last cell of FP32 records (axis_bounds). Last, because the
+  // docking kernel reads the fields above as pairs from the constant bank:
+  // with these three after mz, 20,000 screening ligands took 1.1% longer, 8 of
+  // 256 atoms on 32 lanes 11%.
+  float kx, ky, kz;
 };
 
 // The upper box bound and the last cell of an axis of n points as floats,
