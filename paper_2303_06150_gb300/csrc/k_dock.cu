@@ -652,17 +652,24 @@ int dock_pick_lanes(const int32_t* h_atom_off, const int32_t* h_rot_off, int L, 
   constexpr double kRestart = 2000.;   // cost of a restart outside its samples
   constexpr int kSms = 152;            // of the measurements
   if ((double)L * R > 400. * sms) return 8;   // fills the chip with any ligands
+  // One pass in integers: up to 60,800 ligands come this far, and the same sums
+  // in FP64, once for each shape, took 287 us of one x86 core for 60,000, this
+  // 54 (60,000 rigid ligands, one restart, one rotation, whole call on GB300:
+  // 332 -> 204 us).
+  int most = 0;         // of 4 n_rigid N + 36 passes n (N + 4): below 2^29
+  unsigned swept = 0;   // of n (N + 4), each at most 8,320: below 2^32 up to 1,290 SMs
+  for (int l = 0; l < L; ++l) {
+    const int N = h_atom_off[l + 1] - h_atom_off[l], n = h_rot_off[l + 1] - h_rot_off[l];
+    const int bonds = n * (N + 4), cost = 4 * n_rigid * N + 36 * passes * bonds;
+    most = cost > most ? cost : most;
+    swept += (unsigned)bonds;
+  }
+  const double largest = most / 4., rigid = (double)n_rigid * h_atom_off[L], moving = passes * (swept / 4.);
   int best = 8;
   double best_us = 0.;
   for (const Model& m : kModels) {
     const double slots = 36. * sweep_slots(m.lanes, n_theta, fmt) / sweep_slots(m.lanes, 36, fmt);
-    double work = 0., largest = 0.;
-    for (int l = 0; l < L; ++l) {
-      const double N = h_atom_off[l + 1] - h_atom_off[l], n = h_rot_off[l + 1] - h_rot_off[l];
-      const double rigid = n_rigid * N, moving = passes * n * (N + 4.) / 4.;
-      work += rigid + slots * moving + kRestart;
-      largest = std::max(largest, rigid + 36. * moving);
-    }
+    const double work = rigid + slots * moving + kRestart * L;
     const double us = std::hypot(m.us + m.us_per_cost * largest, work * R / (m.cost_per_us * sms / kSms));
     if (m.lanes == 8 || us < best_us) {
       best = m.lanes;
