@@ -11,7 +11,10 @@
 // independent 256-bit gathers are in flight per moving atom; the wide shapes
 // (a restart per half-warp or warp, for launches too small to fill the chip)
 // also take UT moving atoms at once, since there the chain of loads is the
-// time. Every shape adds in the same order, so results do not depend on it.
+// time. Shapes of 8, 16 and 32 lanes add in the same order, so results do not
+// depend on which of them runs; 2 and 4 lanes (a bucket can be tuned to them)
+// sum the final score in 2 and 4 parts instead of 8, and near-ties between
+// poses can rank another way.
 //
 // Shared memory per CTA: the ligand (centred coordinates + type, bond axes,
 // moving-atom lists) and the current coordinates of every restart, in grid
@@ -622,6 +625,14 @@ int sweep_slots(int G, int n_theta, int fmt) {
   return (n_theta + per - 1) / per * per;
 }
 
+// Length of a sweep's chain of loads: one round trip per chunk, shorter with
+// fewer slots in flight, by about their square root.
+double sweep_chain(int G, int n_theta, int fmt) {
+  const Shape* sh = pick_shape(G, n_theta, fmt, false);
+  const int per = sh->G * sh->SLOTS;
+  return (n_theta + per - 1) / per * std::sqrt((double)sh->SLOTS);
+}
+
 }  // namespace
 
 // Lanes per restart of a plain launch. A launch that fills the chip is
@@ -632,8 +643,9 @@ int sweep_slots(int G, int n_theta, int fmt) {
 // rate) and the shortest taken. Work counts the candidate samples of the
 // rigid stage and of full sweeps of n_theta = 36 slots, (N + 4) / 4 moving
 // atoms a bond (plan_groups' estimate) and a constant per restart for the
-// rest. Constants fitted to launches of 1-20,000 screening, 5-1,000 bimodal
-// and 32-20,000 small ligands on GB300, longest ligand first; measured
+// rest; the chain is the work of the ligand with the most, its sweeps scaled
+// by sweep_chain. Constants fitted to launches of 1-20,000 screening, 5-1,000
+// bimodal and 32-20,000 small ligands on GB300, longest ligand first; measured
 // docking kernel (us), * the one chosen:
 //                        5 ligands   20        80        160       320
 //   screening   8 lanes  303         217       272       483*      702*
@@ -642,6 +654,12 @@ int sweep_slots(int G, int n_theta, int fmt) {
 //   bimodal     8 lanes  547         618       752       922       1087*
 //              16 lanes  221         266*      377*      725*      1391
 //              32 lanes  184*        229       625       1280      2484
+// Other increments, whole calls of 256 restarts, 3 passes (us; in brackets the
+// one chosen while every chain was taken as 36 increments long):
+//   20 of 100-120 atoms, 180 increments   8 lanes [1,715]  16  884   32  870*
+//   40 of 24-52 atoms, 180 increments     8 lanes  [629]   16  302*  32  352
+//   80 of 24-52 atoms, 120 increments     8 lanes  [510]   16  403*  32  452
+//   160 of 100-120 atoms, 12 increments   8 lanes   817*   16 [972]  32 1,584
 int dock_pick_lanes(const int32_t* h_atom_off, const int32_t* h_rot_off, int L, int R, int n_rigid, int n_theta,
                     int passes, int fmt, int sms) {
   struct Model {
@@ -658,18 +676,22 @@ int dock_pick_lanes(const int32_t* h_atom_off, const int32_t* h_rot_off, int L, 
   // 332 -> 204 us).
   int most = 0;         // of 4 n_rigid N + 36 passes n (N + 4): below 2^29
   unsigned swept = 0;   // of n (N + 4), each at most 8,320: below 2^32 up to 1,290 SMs
+  int most_swept = 0;
   for (int l = 0; l < L; ++l) {
     const int N = h_atom_off[l + 1] - h_atom_off[l], n = h_rot_off[l + 1] - h_rot_off[l];
     const int bonds = n * (N + 4), cost = 4 * n_rigid * N + 36 * passes * bonds;
     most = cost > most ? cost : most;
+    most_swept = bonds > most_swept ? bonds : most_swept;
     swept += (unsigned)bonds;
   }
-  const double largest = most / 4., rigid = (double)n_rigid * h_atom_off[L], moving = passes * (swept / 4.);
+  const double rigid = (double)n_rigid * h_atom_off[L], moving = passes * (swept / 4.);
   int best = 8;
   double best_us = 0.;
   for (const Model& m : kModels) {
     const double slots = 36. * sweep_slots(m.lanes, n_theta, fmt) / sweep_slots(m.lanes, 36, fmt);
+    const double longer = sweep_chain(m.lanes, n_theta, fmt) / sweep_chain(m.lanes, 36, fmt) - 1.;
     const double work = rigid + slots * moving + kRestart * L;
+    const double largest = most / 4. + 36. * longer * passes * (most_swept / 4.);
     const double us = std::hypot(m.us + m.us_per_cost * largest, work * R / (m.cost_per_us * sms / kSms));
     if (m.lanes == 8 || us < best_us) {
       best = m.lanes;

@@ -46,7 +46,8 @@ def _estimate(atoms, rot, R, n_rigid, n_theta, passes):
         slots, chunks = _sweep(G, n_theta)
         s36, c36 = _sweep(G, 36)
         work = (rigid + 36 * G * slots * chunks / (G * s36 * c36) * moving + 2000).sum()
-        chain = (rigid + 36 * moving).max()
+        longer = chunks * slots ** 0.5 / (c36 * s36 ** 0.5) - 1
+        chain = (rigid + 36 * moving).max() + 36 * longer * moving.max()
         out[G] = math.hypot(us + per_cost * chain, work * R / rate)
     return out
 
@@ -65,6 +66,17 @@ def test_one_pass_chooses_what_the_sums_choose(pick):
         assert est[got] <= min(est.values()) * (1 + 1e-9)
         seen.add(got)
     assert seen == {8, 16, 32}
+
+
+# measured launches (256 restarts, 24 rotations, 3 passes) whose fastest lanes are well ahead of the others
+@pytest.mark.parametrize("ligands,atoms,rot,n_theta,fastest", [
+    (40, (24, 52), (2, 10), 180, (16, 32)), (20, (24, 52), (2, 10), 180, (16, 32)), (80, (24, 52), (2, 10), 120, (16, 32)),
+    (20, (100, 120), (20, 30), 180, (16, 32)), (5, (100, 120), (20, 30), 180, (32,)), (40, (100, 120), (20, 30), 120, (16, 32)),
+    (160, (100, 120), (20, 30), 12, (8,)), (160, (24, 52), (2, 10), 12, (8,)), (80, (12, 24), (1, 3), 180, (16,))])
+def test_other_increments(pick, ligands, atoms, rot, n_theta, fastest):
+    rng = np.random.default_rng(0)
+    assert pick(rng.integers(atoms[0], atoms[1] + 1, ligands), rng.integers(rot[0], rot[1] + 1, ligands), 256, 24,
+                n_theta, 3)() in fastest
 
 
 def test_host_time_of_a_large_library(pick):
