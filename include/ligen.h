@@ -250,7 +250,9 @@ int ligen_dock_batch(const ligen_ligands_t* ligands, const ligen_grid_t* grid,
  * grows with the largest grid, not with the number of sites. Two sets, with
  * consecutive sites overlapping on internal streams joined back to `stream`,
  * for plain greedy calls on device memory without stage_ms; one set
- * otherwise, and where two would not fit the workspace limit or the memory.
+ * otherwise, where two would not fit the workspace limit or the free memory,
+ * and where a captured call would have to allocate the second. Both stay
+ * allocated, like every workspace, until ligen_release_workspaces.
  * Outputs are site-major: site g's scores start at out_scores + g * L * K,
  * its poses at out_poses + g * K * (7 * L + total rotatable bonds); trace,
  * top_restart and scores_f64 (when given) are likewise [n_sites][...] with

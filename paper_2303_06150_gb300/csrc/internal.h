@@ -169,6 +169,19 @@ struct RescoreArgs {
   unsigned* check;          // checked builds: first out-of-range code, else NULL
 };
 
+// Bytes a workspace grows to for a call that needs `bytes`, under a limit (0:
+// none), and whether a workspace of `cap` bytes (given back first) can, with
+// `free` bytes on the device, allocated in pages of 2 MB.
+inline size_t workspace_want(size_t bytes, size_t limit) {
+  const size_t want = bytes + bytes / 8 + (1 << 20);
+  return limit && want > limit ? limit : want;
+}
+inline bool workspace_fits(size_t bytes, size_t cap, size_t free, size_t limit) {
+  if (limit && bytes > limit) return false;
+  const size_t page = 2 << 20;
+  return bytes <= cap || (workspace_want(bytes, limit) + page - 1) / page * page <= free + cap / page * page;
+}
+
 // Grid records in format `fmt` (RecFormat). beside_pack: launched right
 // after launch_pack on the same stream, it may start with the packer (neither
 // reads what the other writes) and ends after it: scoring 3 poses of 5,001

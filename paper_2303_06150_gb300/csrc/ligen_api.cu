@@ -108,8 +108,7 @@ int get_workspace(cudaStream_t s, size_t bytes, char** out) {
       w.base = nullptr;
       w.cap = 0;
     }
-    size_t want = bytes + bytes / 8 + (1 << 20);
-    if (limit && want > limit) want = limit;
+    const size_t want = workspace_want(bytes, limit);
     cudaError_t e = cudaMalloc(&w.base, want);
     if (e != cudaSuccess) {
       cudaGetLastError();
@@ -120,6 +119,30 @@ int get_workspace(cudaStream_t s, size_t bytes, char** out) {
   }
   *out = w.base;
   return LIGEN_OK;
+}
+
+// Whether get_workspace would succeed, without giving up what the stream has:
+// it synchronises and frees the old workspace before it allocates, and a
+// stream that is being captured cannot do either. The device is asked only
+// where the workspace would have to grow.
+bool workspace_available(cudaStream_t s, size_t bytes) {
+  int dev = 0;
+  if (cudaGetDevice(&dev) != cudaSuccess) return false;
+  size_t cap = 0;
+  {
+    std::lock_guard<std::mutex> lk(g_ws_mu);
+    const auto it = g_ws.find({dev, s});
+    if (it != g_ws.end()) cap = it->second.cap;
+  }
+  if (bytes <= cap) return workspace_fits(bytes, cap, 0, g_ws_limit.load());
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  size_t free = 0, total = 0;
+  if (cudaStreamIsCapturing(s, &cs) != cudaSuccess || cs != cudaStreamCaptureStatusNone ||
+      cudaMemGetInfo(&free, &total) != cudaSuccess) {
+    cudaGetLastError();
+    return false;
+  }
+  return workspace_fits(bytes, cap, free, g_ws_limit.load());
 }
 
 // ------------------------------------------------------------ checking --
@@ -1099,7 +1122,8 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
   // another docks, and its first CTAs fill the SMs that the other's last
   // ligands leave idle (301 screening ligands x 12 sites: 8.27 ms one after
   // another, 7.50 ms). Device memory only, plain greedy launches, no stage
-  // times; dropped where it would exceed the workspace limit or the memory.
+  // times; dropped where it would exceed the workspace limit or the free
+  // memory, or would have to be allocated while the stream is captured.
   struct SiteSet {
     size_t coef, rs, rk, rc, tmp_poses, tmp_top, s64, table;
   } set[2];
@@ -1118,8 +1142,7 @@ static int dock_impl(const ligen_ligands_t* ligands, const ligen_grid_t* grids, 
       set[1].s64 = ar.take(8 * (size_t)L * K);
       if (o_table == o_coef) set[1].table = set[1].coef;   // else both write the same table
     }
-    const size_t limit = g_ws_limit.load();
-    overlap = !limit || ar.used <= limit;
+    overlap = workspace_available(s, ar.used);
   }
   rc = LIGEN_ERR_OOM;
   if (overlap) rc = get_workspace(s, ar.used, &ar.base);
