@@ -67,6 +67,13 @@ int space_of(std::initializer_list<const void*> ptrs) {
   return s == -2 ? 0 : s;
 }
 
+// Whether a kernel can store 32-bit values at every one of them (a copy can
+// write at any address).
+bool word_aligned(std::initializer_list<const void*> ptrs) {
+  for (const void* p : ptrs)
+    if (reinterpret_cast<uintptr_t>(p) & 3) return false;
+  return true;
+}
 
 // ------------------------------------------------------------ workspace --
 struct Workspace {
@@ -1856,27 +1863,28 @@ int ligen_pack_ligands(const ligen_ligands_t* ligands, int32_t n_channels, uint3
   Arena ar;
   LigandPlan lp;
   plan_ligands(ar, ligands, sh, lhost == 1, &lp);
-  // device outputs are written in place, host outputs through the workspace
-  const size_t o_status = ohost && status ? ar.take(4 * (size_t)L) : 0;
-  const size_t o_bucket = ohost && bucket ? ar.take(4 * (size_t)L) : 0;
-  const size_t o_bits = ohost && frag_bits ? ar.take(32 * (size_t)sh.rot) : 0;
-  const size_t o_axis = ohost && axis ? ar.take(8 * (size_t)sh.rot) : 0;
+  // device outputs are written in place, host and unaligned ones through the workspace
+  const bool copy = ohost || !word_aligned({frag_bits, axis, bucket, status});
+  const size_t o_status = copy && status ? ar.take(4 * (size_t)L) : 0;
+  const size_t o_bucket = copy && bucket ? ar.take(4 * (size_t)L) : 0;
+  const size_t o_bits = copy && frag_bits ? ar.take(32 * (size_t)sh.rot) : 0;
+  const size_t o_axis = copy && axis ? ar.take(8 * (size_t)sh.rot) : 0;
   if (ar.used && (rc = get_workspace(s, ar.used, &ar.base)) != LIGEN_OK) return rc;
   LigandsDev lig;
   if ((rc = stage_ligands(ar, ligands, sh, lp, s, &lig)) != LIGEN_OK) return rc;
   Packed pk{};
-  pk.status = ohost && status ? ar.at<int32_t>(o_status) : status;
-  pk.bucket = ohost && bucket ? ar.at<int32_t>(o_bucket) : bucket;
-  pk.fbits = ohost && frag_bits ? ar.at<uint32_t>(o_bits) : frag_bits;
-  pk.axis = ohost && axis ? ar.at<int32_t>(o_axis) : axis;
+  pk.status = copy && status ? ar.at<int32_t>(o_status) : status;
+  pk.bucket = copy && bucket ? ar.at<int32_t>(o_bucket) : bucket;
+  pk.fbits = copy && frag_bits ? ar.at<uint32_t>(o_bits) : frag_bits;
+  pk.axis = copy && axis ? ar.at<int32_t>(o_axis) : axis;
   LG_CUDA(launch_pack(lig, n_channels, pk, sh.max_atoms, s));
-  if (!ohost) return LIGEN_OK;
-  const cudaMemcpyKind k = cudaMemcpyDeviceToHost;
+  if (!copy) return LIGEN_OK;
+  const cudaMemcpyKind k = ohost ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice;
   if (frag_bits && sh.rot) LG_CUDA(cudaMemcpyAsync(frag_bits, pk.fbits, 32 * (size_t)sh.rot, k, s));
   if (axis && sh.rot) LG_CUDA(cudaMemcpyAsync(axis, pk.axis, 8 * (size_t)sh.rot, k, s));
   if (bucket) LG_CUDA(cudaMemcpyAsync(bucket, pk.bucket, 4 * (size_t)L, k, s));
   if (status) LG_CUDA(cudaMemcpyAsync(status, pk.status, 4 * (size_t)L, k, s));
-  LG_CUDA(cudaStreamSynchronize(s));
+  if (ohost) LG_CUDA(cudaStreamSynchronize(s));
   return LIGEN_OK;
 }
 
@@ -1898,16 +1906,18 @@ int ligen_pack_touch(const ligen_ligands_t* ligands, int32_t n_channels, uint32_
   Arena ar;
   LigandPlan lp;
   plan_ligands(ar, ligands, sh, lhost == 1, &lp);
-  const size_t o_touch = ohost ? ar.take(4 * (size_t)sh.rot) : 0;
+  const bool copy = ohost || !word_aligned({touch});
+  const size_t o_touch = copy ? ar.take(4 * (size_t)sh.rot) : 0;
   if (ar.used && (rc = get_workspace(s, ar.used, &ar.base)) != LIGEN_OK) return rc;
   LigandsDev lig;
   if ((rc = stage_ligands(ar, ligands, sh, lp, s, &lig)) != LIGEN_OK) return rc;
   Packed pk{};
-  pk.touch = ohost ? ar.at<uint32_t>(o_touch) : touch;
+  pk.touch = copy ? ar.at<uint32_t>(o_touch) : touch;
   LG_CUDA(launch_pack(lig, n_channels, pk, sh.max_atoms, s));
-  if (!ohost) return LIGEN_OK;
-  LG_CUDA(cudaMemcpyAsync(touch, pk.touch, 4 * (size_t)sh.rot, cudaMemcpyDeviceToHost, s));
-  LG_CUDA(cudaStreamSynchronize(s));
+  if (!copy) return LIGEN_OK;
+  LG_CUDA(cudaMemcpyAsync(touch, pk.touch, 4 * (size_t)sh.rot, ohost ? cudaMemcpyDeviceToHost : cudaMemcpyDeviceToDevice,
+                          s));
+  if (ohost) LG_CUDA(cudaStreamSynchronize(s));
   return LIGEN_OK;
 }
 
