@@ -11,7 +11,11 @@
 // divided out once per thread. Measured on GB300, 96^3 x 8: FP32 63 -> 40.5 us
 // (6.1 TB/s), FP16 66 -> 35 us, against one thread per record with 64-bit
 // divisions and eight loads each. With a block's threads inside one row, a
-// call with a 2 x 1500 x 1500 x 1 grid took 179 us, now 25.
+// call with a 2 x 1500 x 1500 x 1 grid took 179 us, now 23. A plane that
+// fits a block several times over gives the spare threads the marches above it
+// (2 x 2 x 4000001 x 1, whole call: 242 us without, 50), two cells each where
+// it is narrower than a warp (with 12, 78 us: a warp's stores lie 384 bytes
+// apart).
 #include "internal.h"
 
 namespace ligen {
@@ -42,17 +46,27 @@ __device__ __forceinline__ unsigned pack16(float a, float b) {   // rounded to n
   }
 }
 
-// Block: (tile of the plane's (x, y, channel) columns, march). 16-bit
-// record grids have rec_cells(n) = n cells per axis: corners past the last
-// node repeat it (the padding layers of the clamp-free sampler).
-template <int FMT>
+// Block: (tile of the plane's (x, y, channel) columns, march), or with THIN
+// `per` marches of a plane that fits a block `per` times over. 16-bit record
+// grids have rec_cells(n) = n cells per axis: corners past the last node
+// repeat it (the padding layers of the clamp-free sampler).
+template <int FMT, bool THIN>
 __global__ void __launch_bounds__(kPrepThreads) grid_prep_kernel(const float* __restrict__ v, int nx, int ny, int nz,
-                                                                 int nc, unsigned tiles, int march,
+                                                                 int nc, unsigned tiles, int march, int per,
                                                                  void* __restrict__ out) {
   const int cx = rec_cells(nx, FMT), cy = rec_cells(ny, FMT), cz = rec_cells(nz, FMT);
-  const unsigned tile = blockIdx.x % tiles, t = tile * kPrepThreads + threadIdx.x;   // < 2^32 (check_grid)
-  const int z0 = (int)(blockIdx.x / tiles) * march;
+  const unsigned tile = blockIdx.x % tiles;
+  unsigned t = tile * kPrepThreads + threadIdx.x;   // < 2^32 (check_grid)
   const unsigned row = (unsigned)cx * nc;
+  int m = (int)(blockIdx.x / tiles);   // march
+  if constexpr (THIN) {
+    const unsigned sub = t / (row * cy);
+    if (sub >= (unsigned)per) return;
+    t -= sub * (row * cy);
+    m = m * per + (int)sub;
+    if (m >= (cz + march - 1) / march) return;
+  }
+  const int z0 = m * march;
   const int iy = (int)(t / row);
   if (iy >= cy) return;
   const int ix = (int)(t % row / nc), c = (int)(t % row % nc);
@@ -96,10 +110,13 @@ template <int FMT>
 cudaError_t launch_prep(const float* values, int nx, int ny, int nz, int nc, void* rec, bool beside_pack,
                         cudaStream_t s) {
   const size_t cx = rec_cells(nx, FMT), cy = rec_cells(ny, FMT), cz = rec_cells(nz, FMT);
-  const size_t tiles = (cx * cy * nc + kPrepThreads - 1) / kPrepThreads;
+  const size_t columns = cx * cy * nc;
+  const size_t tiles = (columns + kPrepThreads - 1) / kPrepThreads;
+  const size_t per = columns < kPrepThreads ? kPrepThreads / columns : 1;
   const size_t full = tiles * cz / kPrepBlocks;
-  const size_t march = full < 2 ? 2 : full < kPrepMarch ? full : kPrepMarch;
-  const size_t blocks = tiles * ((cz + march - 1) / march);
+  const size_t march = full < 2 || columns < 32 ? 2 : full < kPrepMarch ? full : kPrepMarch;
+  const size_t marches = (cz + march - 1) / march;
+  const size_t blocks = tiles * ((marches + per - 1) / per);
   cudaLaunchConfig_t cfg{};
   cfg.gridDim = dim3((unsigned)blocks);
   cfg.blockDim = dim3(kPrepThreads);
@@ -109,7 +126,8 @@ cudaError_t launch_prep(const float* values, int nx, int ny, int nz, int nc, voi
   at.val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = &at;
   cfg.numAttrs = beside_pack ? 1 : 0;
-  return cudaLaunchKernelEx(&cfg, grid_prep_kernel<FMT>, values, nx, ny, nz, nc, (unsigned)tiles, (int)march, rec);
+  return cudaLaunchKernelEx(&cfg, per > 1 ? grid_prep_kernel<FMT, true> : grid_prep_kernel<FMT, false>, values, nx, ny,
+                            nz, nc, (unsigned)tiles, (int)march, (int)per, rec);
 }
 
 }  // namespace
