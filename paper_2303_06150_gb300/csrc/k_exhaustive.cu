@@ -395,25 +395,31 @@ __global__ void __launch_bounds__(kExThreads, MINB) exhaustive_kernel(const Dock
 // shortens it to b / C, at about 14 ns per rotation, atom and square root of
 // its combinations (an atom's table entries lie between 1 and all
 // combinations; the geometric mean). The C with the smallest sum is taken,
-// no more than there are rotations. Where all rotations fit kExSmall entries
-// the chain is short whatever C. Measured on GB300, whole calls (us; 1,000,
+// no more than there are rotations; where all rotations fit kExSmall entries
+// the chain is short whatever C. One CTA takes the small build while all
+// rotations fit kExTable entries: its time is then its fixed work, of which the
+// small build runs eight CTAs to the other's three (two bonds at 180 degrees,
+// 5,000 x 16: 1,243 rebuilt, 1,887 and 1,268 us with the large and the small
+// build; one bond at 90 degrees 1,090, 1,624 and 1,016). Measured on GB300,
+// whole calls (us; 1,000,
 // 100, 50 or 5,000 ligands of 8-20 atoms, restarts, 30 degree steps, 24
 // rotations), * the one chosen; "rebuilt" is one CTA per (ligand, restart)
 // with every combination rebuilt:
 //                        rebuilt   C = 1     2       4       8     small build
 //   0 bonds   5,000 x 16     844    1,053   2,041   3,902   8,567     591*
-//   0-1       5,000 x 16   1,644    1,363*  2,534   4,680   9,806     984
+//   0-1       5,000 x 16   1,644    1,363   2,534   4,680   9,806     984*
 //   2         1,000 x 16   4,469      854*  1,078   1,564   2,705     846
 //   2         1,000 x 1      425      268     151*    141     199     473
 //   3         50 x 16      4,035      255     243     254*    331     312
 //   0-3       100 x 1      2,651      236     132      85      64*    404
 cudaError_t launch_exhaustive(const DockArgs& a, const ExWork& w, int sms, cudaStream_t s) {
   const long long items = (long long)a.lig.L * a.R;
-  const bool small = w.entries * a.n_rigid <= kExSmall;
   const double per_cta = 5.6 * (double)items / (3. * sms), chain = 0.014 * a.n_rigid * w.chain;
   int C = 1;
-  for (int c = 2; c <= kExCluster && c <= a.n_rigid && !small; c *= 2)
-    if (per_cta * c + chain / c < per_cta * C + chain / C) C = c;
+  if (w.entries * a.n_rigid > kExSmall)
+    for (int c = 2; c <= kExCluster && c <= a.n_rigid; c *= 2)
+      if (per_cta * c + chain / c < per_cta * C + chain / C) C = c;
+  const bool small = C == 1 && w.entries <= kExSmall && w.entries * a.n_rigid <= kExTable;
   const auto kernel = small ? a.fmt == kRecF32   ? exhaustive_kernel<kRecF32, 8>
                               : a.fmt == kRecF16 ? exhaustive_kernel<kRecF16, 8>
                                                  : exhaustive_kernel<kRecBF16, 8>
