@@ -130,7 +130,6 @@ __device__ inline bool fk_stage(const Packed& pk, int a0, int N, int r0, int n, 
   }
   bad = __any_sync(0xffffffffu, bad);
   __syncwarp();
-  __syncwarp();
   return !bad;
 }
 

@@ -25,8 +25,8 @@
 // the ligand and lays out the table again. launch_exhaustive has the rule.
 // Measured on GB300, 97 ligands of 8-20 atoms and 0-3 bonds, 8 restarts, 30
 // degree steps, whole call: 2,780 us with every combination rebuilt by one
-// CTA per (ligand, restart), 269 us this way (280 with eight CTAs for every
-// call).
+// CTA per (ligand, restart), 173-273 us this way by the seed's library (269
+// where eight CTAs for every call take 280).
 #include <cooperative_groups.h>
 
 #include "../../include/ligen.h"

@@ -599,8 +599,12 @@ __global__ void __launch_bounds__(32, 16) grad_lane_kernel(const GradArgs a) {
     for (int s = 0; s < a.steps; ++s) {
       // Every lane of the group takes the norms and step factors (the same
       // instructions as one lane doing it); the angles go round-robin. Which
-      // squares are fused into their sum is fixed: a refined pose follows
-      // from comparisons of scores, so an ulp here can part two trajectories.
+      // squares are fused into their sum is written out, not left to the
+      // compiler: a refined pose follows from comparisons of scores, so an ulp
+      // here can part two trajectories. Any fixed choice would do as well;
+      // this one (every fourth square of the whole groups of four fused, the
+      // others rounded before they are added) is what an earlier version's
+      // unrolled loop rounded, so that refined poses kept their bits.
       float nt = 0.f, nq = 0.f, nth = 0.f;
 #pragma unroll
       for (int e = 0; e < 3; ++e) nt = __fadd_rn(nt, __fmul_rn(grad[e], grad[e]));
